@@ -31,27 +31,90 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompil
 
 # Device sources compiled again at run time for user-defined models (NVRTC):
 # embedded into the library as string constants, one per file.
-RTC_EMBED = [("kRtcCheck", "check.cuh"), ("kRtcEmDevice", "em_device.cuh"), ("kRtcArgs", "rtc_args.h"),
-             ("kRtcKernel", "rtc_kernel.cuh")]
+FIXED_INC = os.path.join(GEN_DIR, "sdeb_fixed_tables.inc")
+RTC_EMBED = [("kRtcCheck", os.path.join(CSRC, "check.cuh")), ("kRtcFixedTables", FIXED_INC),
+             ("kRtcFixedMath", os.path.join(CSRC, "fixed_math.cuh")),
+             ("kRtcEmDevice", os.path.join(CSRC, "em_device.cuh")), ("kRtcArgs", os.path.join(CSRC, "rtc_args.h")),
+             ("kRtcKernel", os.path.join(CSRC, "rtc_kernel.cuh"))]
 RTC_INC = os.path.join(GEN_DIR, "sdeb_rtc_sources.inc")
+
+# Working precision (bits) of the table generator below.
+_BITS = 200
+
+
+def _sincos_bits(num, den):
+    """(cos, sin) of num/den in [0, 2), scaled by 2^_BITS: the Taylor series in integers."""
+    x = (num << _BITS) // den
+    c = s = k = 0
+    term = 1 << _BITS
+    while term:
+        if k % 2 == 0:
+            c += term if k % 4 == 0 else -term
+        else:
+            s += term if k % 4 == 1 else -term
+        k += 1
+        term = (term * x >> _BITS) // k
+    return c, s
+
+
+def _ln_bits(num, den):
+    """ln(num/den) scaled by 2^_BITS: 2 atanh((num - den) / (num + den))."""
+    z = ((num - den) << _BITS) // (num + den)
+    total, term, k = 0, z, 1
+    while term:
+        total += term // k
+        term = (term * z >> _BITS) * z >> _BITS
+        k += 2
+    return 2 * total
+
+
+def _rounded(v, q):
+    return (v + (1 << (_BITS - q - 1))) >> (_BITS - q)
+
+
+def fixed_tables():
+    """The tables of csrc/fixed_math.cuh: (cos, sin)(j / 256) in Q62 for j = 0 .. 402 (pi/2 is 402.1 / 256; the
+    cosines 2 units up, so that a rotation's rounding leaves none below 0), and (ln c, c), c in Q15 the largest
+    with m c <= 1 for every m below (257 + j) / 512, ln c in Q58."""
+    trig = []
+    for j in range(403):
+        c, s = _sincos_bits(j, 256)
+        trig.append((_rounded(c, 62) + 2, _rounded(s, 62)))
+    log = []
+    for j in range(256):
+        c = (512 << 15) // (257 + j)
+        log.append((_rounded(_ln_bits(c, 1 << 15), 58), c))
+    return trig, log
+
+
+def _write_if_changed(path, content):
+    os.makedirs(os.path.dirname(path), exist_ok=True)
+    if os.path.exists(path):
+        with open(path) as f:
+            if f.read() == content:
+                return
+    with open(path, "w") as f:
+        f.write(content)
+
+
+def generate_fixed_tables():
+    parts = ["// Generated by build.py: tables of fixed_math.cuh.\n#pragma once\nnamespace sdeb {\n"]
+    for name, rows in zip(("kFixedTrig", "kFixedLog"), fixed_tables()):
+        parts.append("static __device__ const __align__(16) unsigned long long %s[%d][2] = {\n" % (name, len(rows)))
+        parts += ["{0x%016xull, 0x%016xull},\n" % row for row in rows]
+        parts.append("};\n")
+    _write_if_changed(FIXED_INC, "".join(parts) + "}  // namespace sdeb\n")
 
 
 def generate_rtc_sources():
     parts = ["// Generated by build.py from csrc/: the device sources of the run-time compiled kernel.\n"]
-    for name, fname in RTC_EMBED:
-        with open(os.path.join(CSRC, fname)) as f:
+    for name, path in RTC_EMBED:
+        with open(path) as f:
             text = f.read()
         if ")SDEBRTC" in text:
-            raise RuntimeError("%s contains the raw-string delimiter" % fname)
+            raise RuntimeError("%s contains the raw-string delimiter" % path)
         parts.append('static const char %s[] = R"SDEBRTC(%s)SDEBRTC";\n' % (name, text))
-    content = "".join(parts)
-    os.makedirs(GEN_DIR, exist_ok=True)
-    if os.path.exists(RTC_INC):
-        with open(RTC_INC) as f:
-            if f.read() == content:
-                return
-    with open(RTC_INC, "w") as f:
-        f.write(content)
+    _write_if_changed(RTC_INC, "".join(parts))
 
 
 def _nvcc():
@@ -97,6 +160,7 @@ def build(force=False, verbose_ptxas=False, jobs=None, checked=False):
         return lib
     os.makedirs(CHECKED_BUILD_DIR if checked else BUILD_DIR, exist_ok=True)
     os.makedirs(GEN_DIR, exist_ok=True)
+    generate_fixed_tables()
     generate_rtc_sources()
     srcs = sources()
     jobs = jobs or min(len(srcs), os.cpu_count() or 4)

@@ -11,6 +11,16 @@
 // and costs nothing.
 #pragma once
 
+#ifdef __CUDACC_RTC__
+// Compiled at run time (NVRTC) for user-defined models, this file first: no
+// host headers.
+typedef unsigned char uint8_t;
+typedef int int32_t;
+typedef unsigned int uint32_t;
+typedef long long int64_t;
+typedef unsigned long long uint64_t;
+#endif
+
 namespace sdeb {
 
 enum CheckSite : unsigned {

@@ -5,27 +5,19 @@
 //     key operand is a constant-bank read shared by all threads.
 //   * Uniforms u = (w + 1/2) 2^-32 (reading of Eq. 3's "uniform over [0,1]"),
 //     in FP32 within one ulp of the exact value.
-//   * Box-Muller (Eq. 3) in FP32 (SFU approximations) and FP64.
+//   * Box-Muller (Eq. 3) in FP32 (SFU approximations) and FP64 (fixed point).
 //   * Two-constant Cody-Waite reduction of a phase to [-pi, pi] before the SFU
 //     sine/cosine (W. J. Cody, W. Waite, "Software Manual for the Elementary
 //     Functions", 1980: x - q C1 - q C2 with C1 + C2 ~ 2 pi).
 //   * Butterfly sums over the G lanes that share an orbit.
 #pragma once
 
-#ifdef __CUDACC_RTC__
-// Compiled at run time (NVRTC) for user-defined models: no host headers.
-typedef unsigned char uint8_t;
-typedef int int32_t;
-typedef unsigned int uint32_t;
-typedef long long int64_t;
-typedef unsigned long long uint64_t;
-#else
+#ifndef __CUDACC_RTC__
 #include <cstdint>
 #include <cuda_runtime.h>
-#endif
 
-#ifndef __CUDACC_RTC__
-#include "check.cuh"  // the run-time compiled path gets it ahead of this header
+#include "check.cuh"  // the run-time compiled path gets these two ahead of this header
+#include "fixed_math.cuh"
 #endif
 
 namespace sdeb {
@@ -205,25 +197,16 @@ __device__ __forceinline__ void box_muller_f32(uint32_t w_first, uint32_t w_seco
     n_sin = a * s;
 }
 
-// FP64, polar form: amp = radius, (c, s) = (cos, sin)(2 pi U2).
+// FP64: the normals themselves in the place of (c, s), with amplitude 1 (the
+// product with the radius is formed in fixed point, fixed_math.cuh).
 __device__ __forceinline__ void box_muller_polar_f64(uint32_t w_first, uint32_t w_second, double &amp,
                                                      double &c, double &s) {
-    const double u1 = uniform_f64(w_first);
-    const double u2 = uniform_f64(w_second);
-    amp = sqrt(-2.0 * log(u1));
-    sincospi(2.0 * u2, &s, &c);
-}
-
-__device__ __forceinline__ void box_muller_f64(uint32_t w_first, uint32_t w_second, double &n_cos,
-                                               double &n_sin) {
-    double amp, c, s;
-    box_muller_polar_f64(w_first, w_second, amp, c, s);
-    n_cos = amp * c;
-    n_sin = amp * s;
+    amp = 1.0;
+    box_muller_fixed(w_first, w_second, c, s);
 }
 
 // The factor box_muller_polar leaves out of the amplitude (FP32: sqrt(2 ln 2);
-// FP64: 1, the amplitude is the radius).
+// FP64: 1), and the normal of an amplitude and its trig value.
 template <typename Real>
 __device__ __forceinline__ constexpr Real bm_amp_unit() { return sizeof(Real) == 4 ? Real(kBmAmpUnitF32) : Real(1); }
 
@@ -248,7 +231,7 @@ __device__ __forceinline__ void box_muller<float>(uint32_t a, uint32_t b, float 
 }
 template <>
 __device__ __forceinline__ void box_muller<double>(uint32_t a, uint32_t b, double &c, double &s) {
-    box_muller_f64(a, b, c, s);
+    box_muller_fixed(a, b, c, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -270,11 +253,11 @@ __device__ __forceinline__ float reduce_phase(float x, float c_comp) {
     return __fsub_rn(__fmaf_rn(-q, kC2, r), c_comp);
 }
 
-// FP64 keeps the phase unreduced; sin/cos are CUDA's double functions.
+// FP64 keeps the phase unreduced; its sine and cosine reduce it in fixed point.
 __device__ __forceinline__ double reduce_phase(double x, double c_comp) { return x - c_comp; }
 
 __device__ __forceinline__ void sincos_reduced(float r, float &s, float &c) { sincos_approx_f32(r, s, c); }
-__device__ __forceinline__ void sincos_reduced(double r, double &s, double &c) { sincos(r, &s, &c); }
+__device__ __forceinline__ void sincos_reduced(double r, double &s, double &c) { sincos_fixed(r, s, c); }
 
 __device__ __forceinline__ void sincos_phase(float x, float c_comp, float &s, float &c) {
     sincos_reduced(reduce_phase(x, c_comp), s, c);
@@ -286,7 +269,7 @@ __device__ __forceinline__ void sincos_phase(double x, double c_comp, double &s,
     sincos_reduced(reduce_phase(x, c_comp), s, c);
 }
 
-__device__ __forceinline__ void sincos_phase(double x, double &s, double &c) { sincos(x, &s, &c); }
+__device__ __forceinline__ void sincos_phase(double x, double &s, double &c) { sincos_fixed(x, s, c); }
 
 // ---------------------------------------------------------------------------
 // Explicitly rounded arithmetic: the model increments use these so the
@@ -298,6 +281,12 @@ __device__ __forceinline__ float fma_r(float a, float b, float c) { return __fma
 __device__ __forceinline__ double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_r(double a, double b) { return __dmul_rn(a, b); }
+
+// The normal amp * trig of box_muller_polar's output (FP64: trig, amp is 1).
+__device__ __forceinline__ float polar_normal(float amp, float trig) {
+    return mul_r(mul_r(amp, bm_amp_unit<float>()), trig);
+}
+__device__ __forceinline__ double polar_normal(double, double trig) { return trig; }
 
 // ---------------------------------------------------------------------------
 // Sums over the G consecutive lanes of one orbit.  With a butterfly every

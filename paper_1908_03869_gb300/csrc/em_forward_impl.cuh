@@ -194,14 +194,12 @@ __device__ __forceinline__ void em_step_noise(M &model, Real (&x)[M::U][P], Real
                 if constexpr (M::kDelayedComp) accumulate_delayed(x[c][i], cp[c][i], inc[c]);
                 else accumulate(x[c][i], cp[c][i], inc[c]);
             }
-            if constexpr (RECORD) rec->z[i] = mul_r(mul_r(amp[noise_pair<P>(i)], bm_amp_unit<Real>()), trig[i]);
+            if constexpr (RECORD) rec->z[i] = polar_normal(amp[noise_pair<P>(i)], trig[i]);
         }
     } else {
 #pragma unroll
-        for (int j = 0; j < kNoisePairs<P>; ++j) amp[j] = mul_r(amp[j], bm_amp_unit<Real>());
-#pragma unroll
         for (int i = 0; i < P; ++i) {
-            const Real z = mul_r(amp[noise_pair<P>(i)], trig[i]);
+            const Real z = polar_normal(amp[noise_pair<P>(i)], trig[i]);
             Real inc[M::U];
             model.incr(i, x, red, z, inc);
 #pragma unroll

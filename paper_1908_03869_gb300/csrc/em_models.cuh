@@ -126,7 +126,10 @@ struct KuramotoLane {
     // The scalar noise strength g sqrt(dt) times a Box-Muller amplitude (and
     // the factor the polar form leaves out), once per pair; the increment is
     // then f dt + (g sqrt(dt) amp) trig.
-    __device__ __forceinline__ Real noise_scaled(Real amp) const { return mul_r(gsq_bm, amp); }
+    __device__ __forceinline__ Real noise_scaled(Real amp) const {
+        if constexpr (sizeof(Real) == 8) return gsq_bm;  // FP64: amp is 1
+        else return mul_r(gsq_bm, amp);
+    }
 
     __device__ __forceinline__ void incr_split(int i, const Real (&red)[NR], Real amp_scaled, Real trig,
                                                Real (&inc)[U]) const {

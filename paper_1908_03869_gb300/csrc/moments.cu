@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kMomBlock) state_moments_partial(const Real *f
 // lanes (G a power of two, G >= n up to 32) takes one orbit at a time: each
 // lane sums cos and sin of components lig, lig + G, ... in the frame's
 // precision (FP32: the phase reduced to [-pi, pi] and the special-function
-// unit; FP64: CUDA's double sincos), the group adds them by a butterfly, and
+// unit; FP64: fixed point), the group adds them by a butterfly, and
 // the group's first lane forms r in FP64 and accumulates it.  Every group
 // runs the same number of iterations, so the shuffles always have the whole
 // warp.

@@ -65,6 +65,10 @@ std::string assemble(const sdeb_problem &pb, const char *user_source) {
     std::string src = prelude;
     src += kRtcCheck;
     src += "\n";
+    src += kRtcFixedTables;
+    src += "\n";
+    src += kRtcFixedMath;
+    src += "\n";
     src += kRtcEmDevice;
     src += "\n";
     src += kRtcArgs;

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kFitnessBlock) swarm_fitness_kernel(const Real
             double C = 0.0, S = 0.0;
             for (int32_t j = 0; j < n; ++j) {
                 double s, c;
-                sincos((double)th[j], &s, &c);
+                sincos_fixed((double)th[j], s, c);
                 C += c;
                 S += s;
             }
