@@ -80,7 +80,8 @@ __device__ __forceinline__ void sincos_quarter(uint64_t f, uint64_t &c, uint64_t
     const uint64_t rho = mul_top(f, 0x6487ED5110B4611AULL);  // pi/2 in Q62
     const uint32_t j = (uint32_t)(rho >> 53);
     const uint64_t d = (rho << 3) & 0x00FFFFFFFFFFFFFFULL;
-    const uint32_t dh = (uint32_t)((d + 0x1000000u) >> 25);         // d 2^39
+    // d 2^39, rounded, kept below 2^31 (d just under a table step rounds up to it, and z would be 2^32)
+    const uint32_t dh = min((uint32_t)((d + 0x1000000u) >> 25), 0x7FFFFFFFu);
     const uint32_t z = (uint32_t)(((uint64_t)dh * dh) >> 30);       // d^2 2^48 (< 2^32: d < 2^-8)
     const uint32_t a = __umulhi(z, 0xAAAAAAABu);                    // d^2/6 2^50
     const uint32_t b = __umulhi(__umulhi(a, z), 0x0CCCCCCDu) >> 16;  // d^4/120 2^50
