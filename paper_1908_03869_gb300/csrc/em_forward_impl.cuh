@@ -12,6 +12,7 @@
 namespace sdeb {
 
 constexpr int kForwardBlock = 128;
+constexpr int kNumSms = 152;
 
 // Loads / stores of a lane's units: component c of unit j is row[c*units + j].
 // Full, 16-byte aligned runs use 16-byte vector accesses.
@@ -64,45 +65,66 @@ __device__ __forceinline__ void store_units(Real *row, int units, int u0, const 
 }
 
 // Coupling-sum reducers.  WarpGroupSum<G>: butterfly over the G lanes of an
-// orbit inside one warp.  TeamSum<NW>: an orbit spread over the NW warps of
-// the whole thread block -- warp butterflies, then the NW partial sums
-// exchanged through shared memory (double-buffered, one barrier per call) and
-// added in warp order, so every lane gets bit-identical totals.
+// orbit inside one warp, in the given type or, for models with fixed-point
+// sums (FP64 phases), in 64-bit integers: exact, so the totals are the same
+// bits for every layout.  `bad` becomes true in every lane of an orbit that
+// has a lane with a non-finite phase.
 template <int G>
 struct WarpGroupSum {
+    static constexpr bool kFixedSums = true;
     template <typename Real, int NR>
     __device__ __forceinline__ void operator()(Real (&r)[NR]) const {
 #pragma unroll
         for (int q = 0; q < NR; ++q) r[q] = group_sum<G>(r[q]);
     }
+    __device__ __forceinline__ void fixed(int64_t (&r)[2], bool &bad) const {
+#pragma unroll
+        for (int off = 1; off < G; off <<= 1) {
+            r[0] += __shfl_xor_sync(0xffffffffu, (long long)r[0], off);
+            r[1] += __shfl_xor_sync(0xffffffffu, (long long)r[1], off);
+        }
+        if constexpr (G > 1) {
+            const unsigned all = __ballot_sync(0xffffffffu, bad);
+            bad = ((all >> (threadIdx.x & 31 & ~(G - 1))) & (0xffffffffu >> (32 - G))) != 0;
+        }
+    }
 };
 
-template <int NW, typename Real>
-struct TeamSum {
-    Real *buf;  // shared memory, [2][NW][NRMAX]
+// TeamFixedSum<NW>: an orbit on the NW warps of the whole thread block, for
+// the fixed-point sums: warp butterflies, then the warps' partials exchanged
+// through shared memory (double-buffered, one barrier a call).
+template <int NW>
+struct TeamFixedSum {
+    static constexpr bool kFixedSums = true;
+    longlong2 *buf;  // shared memory, [2][NW]
+    int *bad_buf;    // shared memory, [2][NW]
     int flip;
-    static constexpr int NRMAX = 2;
-    template <int NR>
-    __device__ __forceinline__ void operator()(Real (&r)[NR]) {
-        static_assert(NR <= NRMAX, "TeamSum holds at most NRMAX sums");
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        Real *slot = buf + flip * NW * NRMAX;
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-            r[q] = group_sum<32>(r[q]);
-            if (lane == 0) slot[warp * NRMAX + q] = r[q];
+    __device__ __forceinline__ void fixed(int64_t (&r)[2], bool &bad) {
+        WarpGroupSum<32>().fixed(r, bad);
+        const int warp = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0) {
+            buf[flip * NW + warp] = make_longlong2(r[0], r[1]);
+            bad_buf[flip * NW + warp] = bad;
         }
         __syncthreads();
+        r[0] = r[1] = 0;
+        bad = false;
 #pragma unroll
-        for (int q = 0; q < NR; ++q) {
-            Real t = slot[q];
-#pragma unroll
-            for (int w = 1; w < NW; ++w) t += slot[w * NRMAX + q];
-            r[q] = t;
+        for (int w = 0; w < NW; ++w) {
+            const longlong2 t = buf[flip * NW + w];
+            r[0] += t.x;
+            r[1] += t.y;
+            bad = bad || bad_buf[flip * NW + w] != 0;
         }
         flip ^= 1;
     }
 };
+
+// Whether model M's coupling sums go through reducer RED in fixed point.
+template <class RED, class = void>
+struct FixedReducer : std::false_type {};
+template <class RED>
+struct FixedReducer<RED, std::void_t<decltype(RED::kFixedSums)>> : std::true_type {};
 
 // The lane's fixed Philox words: round 1 of the noise counters (k, block,
 // orbit, 0) of its blocks without k, formed once per launch.
@@ -173,13 +195,20 @@ __device__ __forceinline__ void em_step_noise(M &model, Real (&x)[M::U][P], Real
                                               RED &reduce, StepRecord<Real, P> *rec = nullptr) {
     constexpr int NRA = M::NR > 0 ? M::NR : 1;
     Real red[NRA];
-    model.prepare(x, cp, u0, units, red);
-    if constexpr (M::NR > 0) reduce(red);
+    if constexpr (M::kFixedSums && FixedReducer<RED>::value) {
+        model.fixed_sums(x[0], u0, units, reduce, red);
+    } else {
+        model.prepare(x, cp, u0, units, red);
+        if constexpr (M::NR > 0) reduce(red);
+    }
     if constexpr (RECORD) {
         rec->sums[0] = red[0];
         rec->sums[1] = red[1];
 #pragma unroll
-        for (int i = 0; i < P; ++i) rec->phase[i] = model.rph[i];
+        for (int i = 0; i < P; ++i) {
+            if constexpr (M::kFixedSums) rec->phase[i] = x[0][i];  // FP64 phases are not reduced
+            else rec->phase[i] = model.rph[i];
+        }
     }
     if constexpr (M::kSplitNoise) {
         Real amp_s[kNoisePairs<P>];
@@ -272,8 +301,12 @@ __device__ __forceinline__ void rk4_stage(M &model, const Real (&at)[M::U][P], c
                                           Real weight, Real frac_next) {
     constexpr int NRA = M::NR > 0 ? M::NR : 1;
     Real red[NRA];
-    model.prepare_stage(at, u0, units, red);
-    if constexpr (M::NR > 0) reduce(red);
+    if constexpr (M::kFixedSums && FixedReducer<RED>::value) {
+        model.fixed_sums(at[0], u0, units, reduce, red);
+    } else {
+        model.prepare_stage(at, u0, units, red);
+        if constexpr (M::NR > 0) reduce(red);
+    }
 #pragma unroll
     for (int i = 0; i < P; ++i) {
         Real inc[M::U];
@@ -342,8 +375,12 @@ __device__ __forceinline__ void implicit_step(M &model, Real (&x)[M::U][P], Real
 #pragma unroll
             for (int i = 0; i < P; ++i) z[c][i] = fma_r(theta, d[c][i], base[c][i]);
         Real red[NRA];
-        model.prepare_stage(z, u0, units, red);
-        if constexpr (M::NR > 0) reduce(red);
+        if constexpr (M::kFixedSums && FixedReducer<RED>::value) {
+            model.fixed_sums(z[0], u0, units, reduce, red);
+        } else {
+            model.prepare_stage(z, u0, units, red);
+            if constexpr (M::NR > 0) reduce(red);
+        }
         Real r[M::U][P];
 #pragma unroll
         for (int i = 0; i < P; ++i) {
@@ -415,7 +452,13 @@ __device__ __forceinline__ void em_forward_body(const ForwardArgs &a) {
     uint32_t to_frame = a.stride - (a.k_begin % a.stride);
     uint32_t to_ckpt = a.ckpt_every ? a.ckpt_every - (a.k_begin % a.ckpt_every) : 0u;
 
-    WarpGroupSum<G> reduce;
+    // an orbit on more than a warp has the thread block to itself
+    std::conditional_t<(G > 32), TeamFixedSum<(G + 31) / 32>, WarpGroupSum<(G > 32 ? 32 : G)>> reduce;
+    if constexpr (G > 32) {
+        __shared__ longlong2 team_sums[2 * (G / 32)];
+        __shared__ int team_bad[2 * (G / 32)];
+        reduce = {team_sums, team_bad, 0};
+    }
     const NoiseLane<P> noise(gorb, u0, a.keys);
     // Steps run in runs that end at the next frame, checkpoint or k_end (and,
     // with the periodic compensation, at the next multiple of kCompPeriod),
@@ -522,13 +565,12 @@ __device__ __forceinline__ void em_forward_body(const ForwardArgs &a) {
 #pragma unroll
         for (int i = 0; i < P; ++i)
             if (u0 + i < units && !isfinite(state_value(x[c][i], cp[c][i]))) bad = true;
-    const unsigned ballot = __ballot_sync(0xffffffffu, bad);
-    const int lane = threadIdx.x & 31;
     unsigned group_bits;
-    if constexpr (G == 32) {
-        group_bits = ballot;
+    if constexpr (G > 32) {
+        group_bits = (unsigned)__syncthreads_or(bad);
     } else {
-        group_bits = (ballot >> (lane & ~(G - 1))) & ((1u << G) - 1u);
+        const unsigned ballot = __ballot_sync(0xffffffffu, bad);
+        group_bits = (ballot >> (threadIdx.x & 31 & ~(G - 1))) & (0xffffffffu >> (32 - G));
     }
     if (active) {
         store_units<Real, U, P>(xrow, units, u0, x);
@@ -560,13 +602,20 @@ template <template <typename, int> class MF, typename Real, int G, int P, int SC
 cudaError_t launch_forward_layout(const ForwardArgs &a, cudaStream_t s) {
     using M = MF<Real, P>;
     const int64_t threads = a.orbits * G;
-    const int64_t grid = (threads + kForwardBlock - 1) / kForwardBlock;
+    int block = kForwardBlock;
+    if constexpr (G > 32) {
+        block = G;
+    } else {
+        // a launch too small for a block on every SM: smaller blocks, so that its warps spread over the SMs
+        while (block > 32 && (threads + block - 1) / block < kNumSms) block /= 2;
+    }
+    const int64_t grid = (threads + block - 1) / block;
     if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     constexpr int minb = kForwardMinBlocks<M, Real, G, P, SCHEME>;
     if constexpr (minb > 0)
-        em_forward_kernel_capped<M, Real, G, P, SCHEME, minb><<<(unsigned)grid, kForwardBlock, 0, s>>>(a);
+        em_forward_kernel_capped<M, Real, G, P, SCHEME, minb><<<(unsigned)grid, block, 0, s>>>(a);
     else
-        em_forward_kernel<M, Real, G, P, SCHEME><<<(unsigned)grid, kForwardBlock, 0, s>>>(a);
+        em_forward_kernel<M, Real, G, P, SCHEME><<<(unsigned)grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -616,6 +665,48 @@ cudaError_t dispatch_tuning_layouts(const ForwardArgs &a, Layout l, cudaStream_t
     SDEB_FORWARD_LAYOUT(4, 16)
     SDEB_FORWARD_LAYOUT(8, 16)
     return dispatch_default_layouts<MF, Real>(a, l, s);
+}
+
+// FP64 phase models: the lanes that a layout's kernel runs on.  The coupling
+// sums are exact in fixed point, so a layout's units can go to more lanes
+// with the same results.  4 units per lane instead of 8 or 16 (registers: five
+// resident blocks instead of three), 2 when that leaves less than two warps for
+// every SM sub-partition, on teams of two or four warps past 64 units.
+// Measured, with the fixed-point sums in both: n = 32, 65536 orbits x 200
+// steps 5.95 ms at 4 units (7.8 at 8 with FP64 sums; the FP64, integer
+// multiply and ALU pipes are then 64 to 75 % busy each); n = 100, 64 orbits x
+// 1000 steps 1.43 ms on teams of two warps (5.5 at 8 units, 16 lanes); n = 4,
+// 1024 orbits x 1000 steps 1.29 ms at 2 units (2.5 at 4).
+inline Layout spread_f64(Layout l, int units, int64_t orbits) {
+    while (l.P > 4 && l.G < 32) l = {l.G * 2, l.P / 2};
+    if (l.P >= 4 && units > 2 && orbits * l.G < (int64_t)kNumSms * 4 * 2 * 32) {
+        l = {1, 2};
+        while (l.G * 2 < units) l.G *= 2;
+    }
+    return l;
+}
+
+template <template <typename, int> class MF>
+cudaError_t dispatch_phase_layouts_f64(const ForwardArgs &a, Layout l, cudaStream_t s) {
+    using Real = double;
+    l = spread_f64(l, a.units, a.orbits);
+    SDEB_FORWARD_LAYOUT(1, 1)
+    SDEB_FORWARD_LAYOUT(1, 2)
+    SDEB_FORWARD_LAYOUT(2, 2)
+    SDEB_FORWARD_LAYOUT(4, 2)
+    SDEB_FORWARD_LAYOUT(8, 2)
+    SDEB_FORWARD_LAYOUT(16, 2)
+    SDEB_FORWARD_LAYOUT(32, 2)
+    SDEB_FORWARD_LAYOUT(64, 2)
+    SDEB_FORWARD_LAYOUT(128, 2)
+    SDEB_FORWARD_LAYOUT(1, 4)
+    SDEB_FORWARD_LAYOUT(2, 4)
+    SDEB_FORWARD_LAYOUT(4, 4)
+    SDEB_FORWARD_LAYOUT(8, 4)
+    SDEB_FORWARD_LAYOUT(16, 4)
+    SDEB_FORWARD_LAYOUT(32, 4)
+    SDEB_FORWARD_LAYOUT(32, 8)
+    return cudaErrorNotSupported;
 }
 
 template <typename Real, int P>

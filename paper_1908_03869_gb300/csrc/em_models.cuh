@@ -38,6 +38,7 @@ template <typename Real, int P, bool PAPER>
 struct KuramotoLane {
     static constexpr int U = 1;
     static constexpr int NR = 2;
+    static constexpr bool kFixedSums = sizeof(Real) == 8;  // fixed_sums: exact sums in 64-bit integers
     static constexpr bool kNoise = true;
     static constexpr bool kSplitNoise = !PAPER;  // one noise strength for every unit
     // FP32: compensation folded into x every kCompPeriod steps (the phase
@@ -106,6 +107,65 @@ struct KuramotoLane {
         }
         red[0] = C;
         red[1] = S;
+    }
+
+    // FP64: sines, cosines and the orbit's sums over the lanes of `reduce`, the
+    // sums as integers in Q54 (at most 256 units: below 2^62; a term's dropped
+    // bits are below 2^-54 of full scale, what an FP64 sum past 1/2 rounds by).
+    // All units go through the fixed-point sequences, in one straight block
+    // with the step's noise for the scheduler; a unit whose phase is outside
+    // their range (its values there mean nothing) is then taken again.
+    template <class RED>
+    __device__ __forceinline__ void fixed_sums(const double (&z)[P], int u0, int units, RED &reduce,
+                                               double (&red)[NR]) {
+        int64_t sum[2] = {0, 0};
+        bool bad = false, in_range = true;
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            const uint32_t hi = (uint32_t)__double2hiint(z[i]);
+            uint64_t c, s;
+            uint32_t c_sign, s_sign;
+            sincos_turn(turn_fraction(hi, (uint32_t)__double2loint(z[i])), c, c_sign, s, s_sign);
+            s_sign ^= hi & 0x80000000u;
+            cs[i] = fixed_to_double(c, 62, c_sign);
+            sn[i] = fixed_to_double(s, 62, s_sign);
+            if (u0 + i < units) {
+                if (phase_fixed(hi)) {
+                    sum[0] += with_sign(c >> 8, c_sign);
+                    sum[1] += with_sign(s >> 8, s_sign);
+                } else {
+                    in_range = false;
+                }
+            }
+        }
+        if (!in_range) {
+#pragma unroll 1
+            for (int i = 0; i < P; ++i) {
+                double zi = 1.0;  // selected, not indexed: the units stay in registers
+#pragma unroll
+                for (int j = 0; j < P; ++j) zi = j == i && u0 + j < units ? z[j] : zi;
+                if (phase_fixed((uint32_t)__double2hiint(zi))) continue;
+                const double2 r = sincos_general(zi);
+#pragma unroll
+                for (int j = 0; j < P; ++j) {
+                    cs[j] = j == i ? r.x : cs[j];
+                    sn[j] = j == i ? r.y : sn[j];
+                }
+                if (isfinite(zi)) {
+                    sum[0] += __double2ll_rn(r.x * 0x1p54);
+                    sum[1] += __double2ll_rn(r.y * 0x1p54);
+                } else {
+                    bad = true;
+                }
+            }
+        }
+        reduce.fixed(sum, bad);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const uint32_t sign = hi32((uint64_t)sum[q]) & 0x80000000u;
+            red[q] = fixed_to_double((uint64_t)with_sign((uint64_t)sum[q], sign), 54, sign);
+            if (bad) red[q] = __longlong_as_double(0x7ff8000000000000LL);
+        }
     }
 
     // f dt = (K/n) dt (S cos x_i - C sin x_i) + omega_i dt, with (K/n) dt S
@@ -193,6 +253,7 @@ template <typename Real, int P, bool MIL>
 struct FhnLane {
     static constexpr int U = 2;
     static constexpr int NR = 1;
+    static constexpr bool kFixedSums = false;
     static constexpr bool kNoise = true;
     static constexpr bool kSplitNoise = false;
     static constexpr bool kDelayedComp = false;
@@ -298,6 +359,7 @@ template <typename Real, int P, int KIND, bool MIL = false>
 struct ScalarLane {
     static constexpr int U = 1;
     static constexpr int NR = 0;
+    static constexpr bool kFixedSums = false;
     static constexpr bool kNoise = KIND != 2;
     static constexpr bool kSplitNoise = false;
     static constexpr bool kDelayedComp = false;

@@ -51,6 +51,12 @@ __device__ __forceinline__ FixedLogEntry fixed_log_table(uint32_t j) {
 
 __device__ __forceinline__ uint32_t hi32(uint64_t v) { return (uint32_t)(v >> 32); }
 
+// v or, with `sign` (0 or 1 << 31), -v.
+__device__ __forceinline__ int64_t with_sign(uint64_t v, uint32_t sign) {
+    const int64_t m = (int64_t)((uint64_t)sign << 32) >> 63;
+    return ((int64_t)v ^ m) - m;
+}
+
 // (a b) >> 64, too small by at most 3, for a, b <= 2^63: the low product is
 // left out and the two cross products add without a carry.  Three wide
 // multiply-adds.
@@ -121,10 +127,11 @@ __device__ __forceinline__ bool phase_fixed(uint32_t hi) { return (hi & 0x7fffff
 
 // |x| / (2 pi) modulo 1 in Q64 (hi, lo: the words of a phase in the range
 // above).  |x| = m 2^-s with s in [32, 63], so the fraction is m times the 96
-// bits of 1/(2 pi) from the one that weighs 2^(s - 64) on, modulo 2^64.
+// bits of 1/(2 pi) from the one that weighs 2^(s - 64) on, modulo 2^64.  (Any
+// other phase gives some value.)
 __device__ __forceinline__ uint64_t turn_fraction(uint32_t hi, uint32_t lo) {
     const uint32_t sh = 1043u - ((hi >> 20) & 0x7ffu);  // s - 32
-    const uint32_t w2 = 0x28BE60DBu >> sh;
+    const uint32_t w2 = __funnelshift_r(0x28BE60DBu, 0u, sh);
     const uint32_t w1 = __funnelshift_r(0x9391054Au, 0x28BE60DBu, sh);
     const uint32_t w0 = __funnelshift_r(0x7F09D5F4u, 0x9391054Au, sh);
     const uint32_t m0 = lo, m1 = (hi & 0xfffffu) | 0x100000u;

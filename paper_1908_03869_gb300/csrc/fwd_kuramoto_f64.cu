@@ -4,8 +4,8 @@
 namespace sdeb {
 
 cudaError_t launch_forward_kuramoto_f64(const ForwardArgs &a, Layout l, cudaStream_t s) {
-    if (a.model == kKuramoto) return dispatch_tuning_layouts<KuramotoScalarLane, double>(a, l, s);
-    if (a.model == kKuramotoPaper) return dispatch_default_layouts<KuramotoPaperLane, double>(a, l, s);
+    if (a.model == kKuramoto) return dispatch_phase_layouts_f64<KuramotoScalarLane>(a, l, s);
+    if (a.model == kKuramotoPaper) return dispatch_phase_layouts_f64<KuramotoPaperLane>(a, l, s);
     return cudaErrorNotSupported;
 }
 
