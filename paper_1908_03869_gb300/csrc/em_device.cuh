@@ -98,6 +98,63 @@ inline PhiloxKeys philox_key_schedule(uint64_t seed) {
 }
 
 // ---------------------------------------------------------------------------
+// Two FP32 values in one 64-bit register pair: one instruction does both
+// (fma.rn.f32x2 and its kin), each half rounded as the scalar instruction
+// rounds it.  Measured: of use where an FP32 kernel is bound by issue slots
+// (the FitzHugh-Nagumo step); the phase kernels, held by the special-function
+// and integer-multiply pipes at the same time, ran from 4 % faster (n = 8) to
+// 5 % slower (n = 128) with it, and stay scalar.
+// ---------------------------------------------------------------------------
+
+struct F2 {
+    unsigned long long v;
+};
+
+__device__ __forceinline__ F2 pack2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ F2 dup2(float a) { return pack2(a, a); }
+__device__ __forceinline__ void unpack2(F2 a, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
+// The units of a lane's pair p.  A noise block's units are paired across its
+// two Box-Muller pairs, (0, 2) and (1, 3): their amplitudes then sit side by
+// side too, without a copy.  A lane of two units has the one pair (0, 1).
+template <int P>
+__device__ __forceinline__ constexpr int pair_lo(int p) { return P == 2 ? 0 : 4 * (p / 2) + (p & 1); }
+template <int P>
+__device__ __forceinline__ constexpr int pair_hi(int p) { return pair_lo<P>(p) + (P == 2 ? 1 : 2); }
+template <int P>
+__device__ __forceinline__ F2 pair_of(const float (&v)[P], int p) { return pack2(v[pair_lo<P>(p)], v[pair_hi<P>(p)]); }
+template <int P>
+__device__ __forceinline__ void set_pair(float (&v)[P], int p, F2 a) {
+    unpack2(a, v[pair_lo<P>(p)], v[pair_hi<P>(p)]);
+}
+
+// ---------------------------------------------------------------------------
 // Uniforms
 // ---------------------------------------------------------------------------
 
@@ -195,6 +252,30 @@ __device__ __forceinline__ void box_muller_f32(uint32_t w_first, uint32_t w_seco
     const float a = amp * kBmAmpUnitF32;
     n_cos = a * c;
     n_sin = a * s;
+}
+
+// Both pairs of a noise block (the same arithmetic, two pairs an
+// instruction): amp[j], trig[2 j] and trig[2 j + 1] are pair j's.
+__device__ __forceinline__ void box_muller_polar_block_f32(const U32x4 &w, float *amp, float *trig) {
+    const F2 t = fma2(pack2(__int2float_rn((int32_t)w.x), __int2float_rn((int32_t)w.z)), dup2(-0x1p-32f),
+                      dup2(-0x1p-33f));
+    F2 poly = fma2(t, dup2(0.360673760222240845f), dup2(0.480898346962987793f));
+    poly = fma2(poly, t, dup2(0.721347520444481703f));
+    poly = fma2(poly, t, dup2(1.44269504088896341f));
+    const F2 y_series = mul2(t, poly);
+    const F2 u = fma2(pack2(__uint2float_rn(w.x), __uint2float_rn(w.z)), dup2(0x1p-32f), dup2(0x1p-33f));
+    const F2 ang = fma2(pack2(__uint2float_rn(w.y), __uint2float_rn(w.w)), dup2(0x1.921fb6p-30f),
+                        dup2(-0x1.921fb6p+1f));
+    float ys[2], uu[2], an[2];
+    unpack2(y_series, ys[0], ys[1]);
+    unpack2(u, uu[0], uu[1]);
+    unpack2(ang, an[0], an[1]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float y = ((j ? w.z : w.x) > 0xFBFFFFFFu) ? ys[j] : -lg2_approx_f32(uu[j]);
+        amp[j] = -sqrt_approx_f32(y);
+        sincos_approx_f32(an[j], trig[2 * j + 1], trig[2 * j]);
+    }
 }
 
 // FP64: the normals themselves in the place of (c, s), with amplitude 1 (the
@@ -331,6 +412,14 @@ __device__ __forceinline__ void accumulate_delayed(float &, float &comp, float i
 __device__ __forceinline__ void renormalize(float &x, float &comp) {
     const float t = __fsub_rn(x, comp);
     comp = __fadd_rn(__fsub_rn(t, x), comp);
+    x = t;
+}
+
+// The same for a pair of units.
+__device__ __forceinline__ void accumulate2(F2 &x, F2 &comp, F2 inc) {
+    const F2 y = sub2(inc, comp);
+    const F2 t = add2(x, y);
+    comp = sub2(sub2(t, x), y);
     x = t;
 }
 

@@ -150,7 +150,7 @@ constexpr int kNoisePairs = P < 4 ? 1 : P / 2;
 template <int P>
 __device__ __forceinline__ constexpr int noise_pair(int i) { return P < 4 ? 0 : i / 2; }
 
-template <typename Real, int P>
+template <typename Real, int P, bool PACKED = false>
 __device__ __forceinline__ void draw_noise(Real (&amp)[kNoisePairs<P>], Real (&trig)[P], uint32_t k, int u0,
                                            const NoiseLane<P> &nl, const PhiloxKeys &keys) {
     if constexpr (P < 4) {
@@ -164,8 +164,12 @@ __device__ __forceinline__ void draw_noise(Real (&amp)[kNoisePairs<P>], Real (&t
 #pragma unroll
         for (int blk = 0; blk < P / 4; ++blk) {
             const U32x4 w = philox4x32_10_fixed(k, nl.r1[blk], keys);
-            box_muller_polar<Real>(w.x, w.y, amp[2 * blk], trig[4 * blk], trig[4 * blk + 1]);
-            box_muller_polar<Real>(w.z, w.w, amp[2 * blk + 1], trig[4 * blk + 2], trig[4 * blk + 3]);
+            if constexpr (PACKED) {
+                box_muller_polar_block_f32(w, amp + 2 * blk, trig + 4 * blk);
+            } else {
+                box_muller_polar<Real>(w.x, w.y, amp[2 * blk], trig[4 * blk], trig[4 * blk + 1]);
+                box_muller_polar<Real>(w.z, w.w, amp[2 * blk + 1], trig[4 * blk + 2], trig[4 * blk + 3]);
+            }
         }
     }
 }
@@ -210,7 +214,23 @@ __device__ __forceinline__ void em_step_noise(M &model, Real (&x)[M::U][P], Real
             else rec->phase[i] = model.rph[i];
         }
     }
-    if constexpr (M::kSplitNoise) {
+    if constexpr (M::kPacked) {
+        static_assert(!RECORD && !M::kDelayedComp, "the packed step is the FitzHugh-Nagumo network's");
+        const typename M::Step2 st = model.step2(red);
+#pragma unroll
+        for (int p = 0; p < P / 2; ++p) {
+            const F2 amp2 = P == 2 ? dup2(amp[0]) : pack2(amp[p / 2 * 2], amp[p / 2 * 2 + 1]);
+            F2 inc[M::U];
+            model.incr2(p, st, x, model.noise_scaled2(amp2), pair_of<P>(trig, p), inc);
+#pragma unroll
+            for (int c = 0; c < M::U; ++c) {
+                F2 x2 = pair_of<P>(x[c], p), cp2 = pair_of<P>(cp[c], p);
+                accumulate2(x2, cp2, inc[c]);
+                set_pair<P>(x[c], p, x2);
+                set_pair<P>(cp[c], p, cp2);
+            }
+        }
+    } else if constexpr (M::kSplitNoise) {
         Real amp_s[kNoisePairs<P>];
 #pragma unroll
         for (int j = 0; j < kNoisePairs<P>; ++j) amp_s[j] = model.noise_scaled(amp[j]);  // includes bm_amp_unit
@@ -248,7 +268,7 @@ __device__ __forceinline__ void em_step(M &model, Real (&x)[M::U][P], Real (&cp)
     static_assert(P == 1 || P == 2 || P % 4 == 0, "a lane holds 1, 2 or a multiple of 4 units");
     Real amp[kNoisePairs<P>], trig[P];
     if constexpr (M::kNoise) {
-        draw_noise<Real, P>(amp, trig, k, u0, nl, keys);
+        draw_noise<Real, P, M::kPacked>(amp, trig, k, u0, nl, keys);
     } else {
 #pragma unroll
         for (int j = 0; j < kNoisePairs<P>; ++j) amp[j] = Real(0);
@@ -431,8 +451,7 @@ __device__ __forceinline__ void em_forward_body(const ForwardArgs &a) {
     (void)SDEB_CHECK(a.check, o >= 0 && o < a.orbits, kChkForwardState, o);
 
     M model;
-    model.load(static_cast<const Real *>(a.params) + o * a.param_stride, u0, units, (Real)a.dt,
-               (Real)sqrt(a.dt));
+    model.load(static_cast<const Real *>(a.params) + o * a.param_stride, u0, units, a.dt, sqrt(a.dt));
 
     Real *xrow = static_cast<Real *>(a.x) + o * n;
     Real x[U][P], cp[U][P];

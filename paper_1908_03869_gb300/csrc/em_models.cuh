@@ -44,6 +44,7 @@ struct KuramotoLane {
     // FP32: compensation folded into x every kCompPeriod steps (the phase
     // the drift reads is x - c, formed anyway by the phase reduction)
     static constexpr bool kDelayedComp = sizeof(Real) == 4;
+    static constexpr bool kPacked = false;
     Real omega_dt[P];         // omega_i dt
     Real live[P];             // 1 for the orbit's units, 0 for padding
     Real gsq[PAPER ? P : 1];  // noise strength times sqrt(dt)
@@ -257,6 +258,16 @@ struct FhnLane {
     static constexpr bool kNoise = true;
     static constexpr bool kSplitNoise = false;
     static constexpr bool kDelayedComp = false;
+    // FP32: two units an instruction (pairs of em_device.cuh), with the noise
+    // inside the bracket that dt multiplies:
+    //   dv = dt (v (sigma / sqrt(dt) N - c - v^2 / 3) + v - w + I + c mean)
+    //   dw = eps dt (v + a - b w)
+    // (Milstein: N + sigma sqrt(dt) (N^2 - 1) / 2 for N).  Ten packed operations
+    // a pair of units.  (Polynomials with dt inside every coefficient take
+    // seven, but the coefficients' roundings then add up over the horizon:
+    // 4.7e-8 from the 64-bit result where this form and the scalar one have 3e-8.)
+    static constexpr bool kPacked = sizeof(Real) == 4 && P > 1;
+    Real kc, kmean, kgsq, kepsdt;
     Real a, b, eps, I, c, gsq, dt, inv_units;
     Real half_gsq2;  // (sigma sqrt(dt))^2 / 2, the Milstein coefficient
 
@@ -269,7 +280,15 @@ struct FhnLane {
             for (int i = 0; i < P; ++i) base[c][i] = x[c][i];
     }
 
-    __device__ __forceinline__ void load(const Real *p, int, int units, Real dt_, Real sqdt) {
+    __device__ __forceinline__ void load(const Real *p, int, int units, double dt64, double sqdt64) {
+        const Real dt_ = (Real)dt64, sqdt = (Real)sqdt64;
+        if constexpr (kPacked) {
+            const double g = (double)p[5] * sqdt64;
+            kgsq = (Real)(g * (double)bm_amp_unit<float>() / dt64);
+            kc = (Real)(-(double)p[4] - (MIL ? 0.5 * g * g / dt64 : 0.0));
+            kmean = (Real)((double)p[4] / units);
+            kepsdt = (Real)((double)p[2] * dt64);
+        }
         a = p[0];
         b = p[1];
         eps = p[2];
@@ -283,6 +302,17 @@ struct FhnLane {
 
     __device__ __forceinline__ void prepare(const Real (&x)[U][P], const Real (&)[U][P], int u0, int units,
                                             Real (&red)[NR]) {
+        if constexpr (kPacked) {
+            if (u0 + P <= units) {
+                F2 s2 = pair_of<P>(x[0], 0);
+#pragma unroll
+                for (int p = 1; p < P / 2; ++p) s2 = add2(s2, pair_of<P>(x[0], p));
+                float lo, hi;
+                unpack2(s2, lo, hi);
+                red[0] = lo + hi;
+                return;
+            }
+        }
         Real sv = 0;
 #pragma unroll
         for (int i = 0; i < P; ++i)
@@ -303,6 +333,25 @@ struct FhnLane {
         inc[0] = fv * dt + gsq * v * N;
         if constexpr (MIL) inc[0] += milstein_multiplicative(half_gsq2, v, N);
         inc[1] = fw * dt;
+    }
+
+    struct Step2 {
+        F2 k0;
+    };
+    __device__ __forceinline__ Step2 step2(const Real (&red)[NR]) const { return Step2{dup2(fma_r(kmean, red[0], I))}; }
+    __device__ __forceinline__ F2 noise_scaled2(F2 amp) const { return mul2(dup2(kgsq), amp); }
+    __device__ __forceinline__ void incr2(int p, const Step2 &st, const Real (&x)[U][P], F2 amp_scaled, F2 trig,
+                                          F2 (&inc)[U]) const {
+        const F2 v = pair_of<P>(x[0], p), w = pair_of<P>(x[1], p);
+        F2 m = fma2(dup2(Real(-1.0 / 3.0)), mul2(v, v), dup2(kc));
+        if constexpr (MIL) {
+            const F2 n = mul2(amp_scaled, trig);
+            m = fma2(n, fma2(n, dup2(Real(0.5) * dt), dup2(Real(1))), m);
+        } else {
+            m = fma2(amp_scaled, trig, m);
+        }
+        inc[0] = mul2(dup2(dt), fma2(v, m, add2(sub2(st.k0, w), v)));
+        inc[1] = mul2(dup2(kepsdt), fma2(dup2(-b), w, add2(v, dup2(a))));
     }
 
     __device__ __forceinline__ void drift_incr(int i, const Real (&x)[U][P], const Real (&red)[NR],
@@ -363,6 +412,7 @@ struct ScalarLane {
     static constexpr bool kNoise = KIND != 2;
     static constexpr bool kSplitNoise = false;
     static constexpr bool kDelayedComp = false;
+    static constexpr bool kPacked = false;
     Real rate, gsq, dt, half_gsq2;
 
     // Base of the ODE schemes' stage states: the state itself.
