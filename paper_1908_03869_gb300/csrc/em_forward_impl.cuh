@@ -90,10 +90,11 @@ struct WarpGroupSum {
     }
 };
 
-// TeamFixedSum<NW>: an orbit on the NW warps of the whole thread block, for
-// the fixed-point sums: warp butterflies, then the warps' partials exchanged
-// through shared memory (double-buffered, one barrier a call).
-template <int NW>
+// TeamFixedSum<NW>: an orbit on the first NW warps of a thread block, for the
+// fixed-point sums: warp butterflies, then the warps' partials exchanged
+// through shared memory (double-buffered, one barrier a call: the block's, or
+// named barrier BAR where the block has other warps).
+template <int NW, int BAR = 0>
 struct TeamFixedSum {
     static constexpr bool kFixedSums = true;
     longlong2 *buf;  // shared memory, [2][NW]
@@ -106,7 +107,8 @@ struct TeamFixedSum {
             buf[flip * NW + warp] = make_longlong2(r[0], r[1]);
             bad_buf[flip * NW + warp] = bad;
         }
-        __syncthreads();
+        if constexpr (BAR == 0) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NW * 32) : "memory");
         r[0] = r[1] = 0;
         bad = false;
 #pragma unroll

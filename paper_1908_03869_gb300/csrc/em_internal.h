@@ -89,12 +89,21 @@ cudaError_t launch_forward_rk4_f32(const ForwardArgs &a, Layout l, cudaStream_t 
 cudaError_t launch_forward_rk4_f64(const ForwardArgs &a, Layout l, cudaStream_t s);
 cudaError_t launch_forward_implicit_f32(const ForwardArgs &a, Layout l, cudaStream_t s);
 cudaError_t launch_forward_implicit_f64(const ForwardArgs &a, Layout l, cudaStream_t s);
+// Few orbits of the phase models (Euler-Maruyama): cudaErrorNotSupported, and
+// nothing launched, when the launch is not small enough, keeps checkpoints or
+// has another layout than the default one.
+cudaError_t launch_forward_split_f32(const ForwardArgs &a, Layout l, cudaStream_t s);
+cudaError_t launch_forward_split_f64(const ForwardArgs &a, Layout l, cudaStream_t s);
 
 // The forward launch of a problem: Runge-Kutta, implicit, phase models or the others.
 inline cudaError_t launch_forward_any(const ForwardArgs &a, Layout l, bool fp64, cudaStream_t s) {
     if (a.rk4) return fp64 ? launch_forward_rk4_f64(a, l, s) : launch_forward_rk4_f32(a, l, s);
     if (a.implicit) return fp64 ? launch_forward_implicit_f64(a, l, s) : launch_forward_implicit_f32(a, l, s);
     const bool phase = a.model == kKuramoto || a.model == kKuramotoPaper;
+    if (phase) {
+        const cudaError_t e = fp64 ? launch_forward_split_f64(a, l, s) : launch_forward_split_f32(a, l, s);
+        if (e != cudaErrorNotSupported) return e;
+    }
     if (phase) return fp64 ? launch_forward_kuramoto_f64(a, l, s) : launch_forward_kuramoto_f32(a, l, s);
     return fp64 ? launch_forward_other_f64(a, l, s) : launch_forward_other_f32(a, l, s);
 }
