@@ -248,7 +248,7 @@ cudaError_t launch_split(const ForwardArgs &a, cudaStream_t s) {
 inline bool use_split(const ForwardArgs &a, Layout l, bool fp64) {
     Layout plain{0, 0};
     if (!default_layout(a.units, plain) || plain.G != l.G || plain.P != l.P) return false;
-    if (a.ckpt != nullptr || (!fp64 && a.units > 128)) return false;
+    if (a.ckpt != nullptr || a.nckpt > 0 || (!fp64 && a.units > 128)) return false;
     int64_t lanes = 1;
     while (lanes < a.units && (fp64 || lanes < 32)) lanes *= 2;
     return a.orbits <= (int64_t)kNumSms * 4 * 32 * (fp64 ? 2 : 1) / lanes;
