@@ -10,6 +10,8 @@
 #include <cstdlib>
 #include <new>
 #include <string>
+#include <functional>
+#include <queue>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -58,6 +60,7 @@ struct sdeb_ctx {
     int *d_head = nullptr;
     int32_t ntasks = 0, team_items = 0;
     int grid = 0;
+    bool grid_tuned = false;              // grid_cap is the tuner's choice
     int grid_cap = 1;                     // resident blocks of the batch kernel on this device
     cudaStream_t capture_stream = nullptr;
     cudaGraphExec_t graph = nullptr;
@@ -311,8 +314,45 @@ struct BatchPlan {
     std::vector<BatchItem> items;
     std::vector<BatchTask> tasks;
     std::vector<Layout> inst_layout;   // (lanes per item, units per lane) of every instance
+    std::vector<double> cost;          // of every task, in ns (batch_step_cost)
     int32_t team_items = 0;
 };
+
+// Resident blocks per SM that end a plan soonest, for FP32: its tasks, in
+// their order, on R blocks of every SM, a block's step taking t(R).  More
+// blocks fill an SM's issue slots (first with packed warps, whose steps have
+// more independent work) and stretch the longest chains, which the queue
+// starts first; every R from 1 to 4 is the best one for some batches.  t(R) in
+// ns, fitted to 13 batches at each R (sums within 7 % where the pick is made):
+// team 140, 160, 200, 265, packed warps 410, 530, 640, 785.  Measured at R = 1
+// to 4, n = 2 to 256: 64 orbits of 48 instances to 1e5 steps 33.4, 22.6, 20.4
+// and 25.7 ms; 32 of 27 to 15141 steps 2.03, 2.20, 2.85 and 2.85; 512 of 48
+// to 1e4 steps 37.4, 24.3, 19.9 and 18.5.  (Five blocks a SM, whatever the
+// batch, on 96 registers a thread: 31.2, 2.84 and 19.3.)
+int plan_residency(const BatchPlan &plan, int num_sms, int most) {
+    constexpr double kTeam[4] = {140.0 / 240.0, 160.0 / 240.0, 200.0 / 240.0, 265.0 / 240.0};
+    constexpr double kPacked[4] = {410.0 / 650.0, 530.0 / 650.0, 640.0 / 650.0, 785.0 / 650.0};
+    int best = 1;
+    double best_end = 0.0;
+    for (int r = 1; r <= std::min(4, most); ++r) {
+        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+        double end = 0.0;
+        for (size_t t = 0; t < plan.tasks.size(); ++t) {
+            double done = plan.cost[t] * (plan.tasks[t].kind == kBatchWarps ? kPacked : kTeam)[r - 1];
+            if ((int64_t)free_at.size() >= (int64_t)r * num_sms) {
+                done += free_at.top();
+                free_at.pop();
+            }
+            free_at.push(done);
+            end = std::max(end, done);
+        }
+        if (r == 1 || end < best_end) {
+            best = r;
+            best_end = end;
+        }
+    }
+    return best;
+}
 
 BatchPlan plan_batch(const std::vector<BatchInstance> &inst, double chain_frac, int num_sms) {
     double total_warp_time = 0.0;   // the whole batch in packed warps of 8 units per lane
@@ -440,7 +480,10 @@ BatchPlan plan_batch(const std::vector<BatchInstance> &inst, double chain_frac, 
         tasks.push_back({t, cost});
     }
     std::stable_sort(tasks.begin(), tasks.end(), [](const Costed &a, const Costed &b) { return a.cost > b.cost; });
-    for (const Costed &c : tasks) plan.tasks.push_back(c.task);
+    for (const Costed &c : tasks) {
+        plan.tasks.push_back(c.task);
+        plan.cost.push_back(c.cost);
+    }
     return plan;
 }
 
@@ -463,7 +506,12 @@ sdeb_status upload_plan(sdeb_ctx *c, const BatchPlan &plan) {
     c->ntasks = (int32_t)plan.tasks.size();
     c->team_items = plan.team_items;
     c->inst_layout = plan.inst_layout;
-    c->grid = std::max(1, std::min<int>(c->ntasks, c->grid_cap));
+    int cap = c->grid_cap;
+    if (c->elem == 4 && !c->grid_tuned) {
+        const int sms = std::max(1, c->num_sms);
+        cap = std::min(cap, sms * plan_residency(plan, sms, std::max(1, cap / sms)));
+    }
+    c->grid = std::max(1, std::min<int>(c->ntasks, cap));
     if (c->graph) {
         cudaGraphExecDestroy(c->graph);
         c->graph = nullptr;
@@ -551,9 +599,11 @@ sdeb_status autotune_batch(sdeb_ctx *c, cudaStream_t s) {
     float best_ms = 1e30f;
     bool first = true;
     const int cap = c->grid_cap;
+    c->grid_tuned = true;
     for (double frac : {0.125, 0.18, 0.25, 0.35, 0.5, 0.7, 1.0, 2.0})
-      for (int per_sm : {2, 3, 4, 5}) {
+      for (int per_sm : {1, 2, 3, 4, 5}) {
         if (e != cudaSuccess) break;
+        if (per_sm > 1 && per_sm * c->num_sms > cap) break;
         c->grid_cap = std::min(cap, per_sm * c->num_sms);
         if (upload_plan(c, plan_batch(c->inst, frac, c->num_sms)) != SDEB_OK) {
             e = cudaErrorUnknown;
