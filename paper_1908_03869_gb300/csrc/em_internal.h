@@ -79,6 +79,13 @@ inline bool delayed_compensation(int32_t model, int32_t precision, uint32_t flag
 // dst[i] = x[i] - comp[i] (FP32), count elements, on the stream (aux_kernels.cu).
 cudaError_t launch_state_value(const float *x, const float *comp, int64_t count, float *dst, cudaStream_t s);
 
+// A run's start from its state x (`bytes` of it): copies to frame 0 and
+// checkpoint 0, zeros to the compensations (as many bytes each) and to the
+// orbits' flags; null pointers are left out.  All are whole allocations of
+// the context (aux_kernels.cu).
+cudaError_t launch_state_reset(const void *x, size_t bytes, void *frame0, void *ckpt0, void *comp, void *ckpt_comp,
+                               uint8_t *flags, int64_t orbits, cudaStream_t s);
+
 // Returns cudaSuccess or the launch error; cudaErrorNotSupported when the
 // (model, precision, layout) combination has no instantiation.
 cudaError_t launch_forward_kuramoto_f32(const ForwardArgs &a, Layout l, cudaStream_t s);

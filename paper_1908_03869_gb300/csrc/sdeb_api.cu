@@ -923,13 +923,9 @@ sdeb_status sdeb_set_params(sdeb_ctx *ctx, const void *params, const void *x0, i
     const size_t state_bytes = (size_t)ctx->pb.orbits * ctx->pb.n * ctx->elem;
     cudaError_t e = cudaMemcpyAsync(ctx->d_params, params, ctx->params_bytes, kind, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_x, x0, state_bytes, kind, s);
-    if (e == cudaSuccess && ctx->d_comp) e = cudaMemsetAsync(ctx->d_comp, 0, state_bytes, s);
-    if (e == cudaSuccess && ctx->d_frames)
-        e = cudaMemcpyAsync(ctx->d_frames, ctx->d_x, state_bytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess && ctx->d_ckpt)
-        e = cudaMemcpyAsync(ctx->d_ckpt, ctx->d_x, state_bytes, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess && ctx->d_ckpt_comp) e = cudaMemsetAsync(ctx->d_ckpt_comp, 0, state_bytes, s);
-    if (e == cudaSuccess && ctx->d_flags) e = cudaMemsetAsync(ctx->d_flags, 0, (size_t)ctx->pb.orbits, s);
+    if (e == cudaSuccess)
+        e = launch_state_reset(ctx->d_x, state_bytes, ctx->d_frames, ctx->d_ckpt, ctx->d_comp, ctx->d_ckpt_comp,
+                               ctx->d_flags, ctx->pb.orbits, s);
     if (e == cudaSuccess && on_device == SDEB_MEM_HOST) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         cudaGetLastError();
