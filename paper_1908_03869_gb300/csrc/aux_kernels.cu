@@ -76,9 +76,8 @@ __global__ void state_value_kernel(const float *x, const float *comp, int64_t co
 }
 
 // One pass for what were up to five copies and fills: bound by launches for
-// few orbits (256 orbits of n = 8, 200 steps, FP32, a whole pass: 1.50 to
-// 1.55 times the speed of before the few-orbit kernel without it, 1.70 with
-// it, 49 us) and by memory for many (the state is read once).
+// few orbits (256 orbits of n = 8, 200 steps, FP32: a whole pass 54.9 us with
+// the five, 48.7 with this) and by memory for many (the state is read once).
 __global__ void __launch_bounds__(256) state_reset_kernel(const uint4 *x, int64_t vecs, int tail, uint4 *frame0,
                                                           uint4 *ckpt0, uint4 *comp, uint4 *ckpt_comp, uint8_t *flags,
                                                           int64_t orbits) {
