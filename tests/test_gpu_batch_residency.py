@@ -1,6 +1,5 @@
 """The batch's resident blocks per SM follow its chains: fewer where a few
-long chains decide, more where there is work for every issue slot;
-results are the bits of every instance alone in its batch, or tuned.
+long chains decide, more where there is work for every issue slot.
 """
 import pytest
 import torch
