@@ -16,10 +16,11 @@
 #pragma once
 
 #include "em_forward_impl.cuh"
+#include "split_chunks.h"
 
 namespace sdeb {
 
-constexpr int kSplitSteps = 8;
+constexpr int kSplitSteps = (int)SplitChunks::kSteps;
 
 // Lanes, warps and orbits of a block, and the producers' share: two noise
 // blocks of four normals per producer lane and buffer half keeps them ahead.
@@ -104,8 +105,8 @@ __global__ void __launch_bounds__(SplitShape<G, P>::kThreads) em_split_kernel(co
         produce(0, 0);
         __syncthreads();
         int half = 1;
-        for (uint32_t k = 0; k < steps; k += kSplitSteps, half ^= 1) {
-            if (steps - k > kSplitSteps) produce(k + kSplitSteps, half);
+        for (SplitChunks c(steps); !c.done(); c.next(), half ^= 1) {
+            if (!c.last()) produce(c.from + kSplitSteps, half);
             __syncthreads();
         }
         __syncthreads();
@@ -153,8 +154,8 @@ __global__ void __launch_bounds__(SplitShape<G, P>::kThreads) em_split_kernel(co
     };
     __syncthreads();  // the first half is full
     int half = 0;
-    for (uint32_t k0 = 0; k0 < steps; k0 += kSplitSteps, half ^= 1) {
-        const int count = (int)min((uint32_t)kSplitSteps, steps - k0);
+    for (SplitChunks c(steps); !c.done(); c.next(), half ^= 1) {
+        const int count = (int)c.count();
         Real amp_next[kNoisePairs<P>], z_next[P];
         read(half, 0, amp_next, z_next);
 #pragma unroll 1
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(SplitShape<G, P>::kThreads) em_split_kernel(co
             for (int i = 0; i < P; ++i) z[i] = z_next[i];
             read(half, min(s + 1, kSplitSteps - 1), amp_next, z_next);
             em_step_noise<M, Real, P>(model, x, cp, amp, z, u0, units, reduce);
-            const uint32_t k = a.k_begin + k0 + (uint32_t)s + 1;
+            const uint32_t k = a.k_begin + c.from + (uint32_t)s + 1;
             if constexpr (M::kDelayedComp) {
                 if ((k & (kCompPeriod - 1u)) == 0) renormalize_units(x, cp);
             }
