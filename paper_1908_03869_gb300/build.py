@@ -72,18 +72,30 @@ def _rounded(v, q):
     return (v + (1 << (_BITS - q - 1))) >> (_BITS - q)
 
 
-def fixed_tables():
-    """The tables of csrc/fixed_math.cuh: (cos, sin)(j / 256) in Q62 for j = 0 .. 402 (pi/2 is 402.1 / 256; the
-    cosines 2 units up, so that a rotation's rounding leaves none below 0), and (ln c, c), c in Q15 the largest
-    with m c <= 1 for every m below (257 + j) / 512, ln c in Q58."""
+def _pi_bits():
+    """pi scaled by 2^_BITS (Machin: 16 atan(1/5) - 4 atan(1/239))."""
+    def atan_inv(n):
+        total, term, k = 0, (1 << _BITS) // n, 1
+        while term:
+            total += term // k if k % 4 == 1 else -(term // k)
+            term //= n * n
+            k += 2
+        return total
+    return 16 * atan_inv(5) - 4 * atan_inv(239)
+
+
+def fixed_tables(step=(1, 256), rows=403, q_cos=62, q_sin=62, q_log=58, up=2):
+    """(cos, sin)(j step) in Q(q_cos) and Q(q_sin), j < rows, the cosines `up` units up (of use where rows pass
+    pi/2: a rotation's rounding then leaves none below 0), and (ln c, c), c in Q15 the largest with m c <= 1 for
+    every m below (257 + j) / 512, ln c in Q(q_log)."""
     trig = []
-    for j in range(403):
-        c, s = _sincos_bits(j, 256)
-        trig.append((_rounded(c, 62) + 2, _rounded(s, 62)))
+    for j in range(rows):
+        c, s = _sincos_bits(j * step[0], step[1])
+        trig.append((_rounded(c, q_cos) + up, _rounded(s, q_sin)))
     log = []
     for j in range(256):
         c = (512 << 15) // (257 + j)
-        log.append((_rounded(_ln_bits(c, 1 << 15), 58), c))
+        log.append((_rounded(_ln_bits(c, 1 << 15), q_log), c))
     return trig, log
 
 
@@ -99,7 +111,8 @@ def _write_if_changed(path, content):
 
 def generate_fixed_tables():
     parts = ["// Generated by build.py: tables of fixed_math.cuh.\n#pragma once\nnamespace sdeb {\n"]
-    for name, rows in zip(("kFixedTrig", "kFixedLog"), fixed_tables()):
+    tables = fixed_tables((_pi_bits(), 4096 << _BITS), 1024, 63, 64, 58, 0)
+    for name, rows in zip(("kFixedTrig", "kFixedLog"), tables):
         parts.append("static __device__ const __align__(16) unsigned long long %s[%d][2] = {\n" % (name, len(rows)))
         parts += ["{0x%016xull, 0x%016xull},\n" % row for row in rows]
         parts.append("};\n")

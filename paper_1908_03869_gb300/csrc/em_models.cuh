@@ -120,44 +120,40 @@ struct KuramotoLane {
     __device__ __forceinline__ void fixed_sums(const double (&z)[P], int u0, int units, RED &reduce,
                                                double (&red)[NR]) {
         int64_t sum[2] = {0, 0};
-        bool bad = false, in_range = true;
+        bool bad = false;
+        uint32_t again = 0;
 #pragma unroll
         for (int i = 0; i < P; ++i) {
             const uint32_t hi = (uint32_t)__double2hiint(z[i]);
-            uint64_t c, s;
-            uint32_t c_sign, s_sign;
-            sincos_turn(turn_fraction(hi, (uint32_t)__double2loint(z[i])), c, c_sign, s, s_sign);
-            s_sign ^= hi & 0x80000000u;
-            cs[i] = fixed_to_double(c, 62, c_sign);
-            sn[i] = fixed_to_double(s, 62, s_sign);
-            if (u0 + i < units) {
-                if (phase_fixed(hi)) {
-                    sum[0] += with_sign(c >> 8, c_sign);
-                    sum[1] += with_sign(s >> 8, s_sign);
-                } else {
-                    in_range = false;
-                }
-            }
+            uint32_t next;
+            const uint64_t turn = turn_fraction(hi, (uint32_t)__double2loint(z[i]), next);
+            const Octant o = sincos_octant(turn, next);
+            const uint32_t c_sign = cos_sign(turn), s_sign = sin_sign(turn) ^ (hi & 0x80000000u);
+            octant_to_double(o, c_sign, s_sign, cs[i], sn[i]);
+            const bool in_range = phase_fixed(hi) && !o.tiny, mine = u0 + i < units;
+            again |= mine && !in_range ? 1u << i : 0u;
+            const uint64_t keep = mine && in_range ? ~0ULL : 0ULL, lg = o.c >> 9, sm = o.s >> 10;
+            sum[0] += with_sign((o.swap ? sm : lg) & keep, c_sign);
+            sum[1] += with_sign((o.swap ? lg : sm) & keep, s_sign);
         }
-        if (!in_range) {
+        // rolled: the instruction cache holds little more than the block above
 #pragma unroll 1
-            for (int i = 0; i < P; ++i) {
-                double zi = 1.0;  // selected, not indexed: the units stay in registers
+        for (; again != 0; again &= again - 1) {
+            const int i = __ffs((int)again) - 1;
+            double zi = 0.0;  // selected, not indexed: the units stay in registers
 #pragma unroll
-                for (int j = 0; j < P; ++j) zi = j == i && u0 + j < units ? z[j] : zi;
-                if (phase_fixed((uint32_t)__double2hiint(zi))) continue;
-                const double2 r = sincos_general(zi);
+            for (int j = 0; j < P; ++j) zi = j == i ? z[j] : zi;
+            const double2 r = phase_small((uint32_t)__double2hiint(zi)) ? sincos_small(zi) : sincos_general(zi);
 #pragma unroll
-                for (int j = 0; j < P; ++j) {
-                    cs[j] = j == i ? r.x : cs[j];
-                    sn[j] = j == i ? r.y : sn[j];
-                }
-                if (isfinite(zi)) {
-                    sum[0] += __double2ll_rn(r.x * 0x1p54);
-                    sum[1] += __double2ll_rn(r.y * 0x1p54);
-                } else {
-                    bad = true;
-                }
+            for (int j = 0; j < P; ++j) {
+                cs[j] = j == i ? r.x : cs[j];
+                sn[j] = j == i ? r.y : sn[j];
+            }
+            if (isfinite(zi)) {
+                sum[0] += __double2ll_rn(r.x * 0x1p54);
+                sum[1] += __double2ll_rn(r.y * 0x1p54);
+            } else {
+                bad = true;
             }
         }
         reduce.fixed(sum, bad);

@@ -5,15 +5,16 @@
 // multiply, fma or conversion) against 22 wide 32 x 32 -> 64 multiplies or 64
 // integer adds or shifts.  CUDA's double sincos, log and sqrt are sequences
 // on that one pipe: they were 59 of the 65.6 FP64 instructions per
-// oscillator-step of the Kuramoto kernel.  Here they are integer sequences
-// whose error is below 2^-56 of full scale before the one rounding to
-// double.
+// oscillator-step of the Kuramoto kernel.  Here they are integer sequences,
+// each result rounded to double once; a sine or cosine is within 2^-52 of the
+// exact one relative to itself, however small it is (measured on the host
+// against 64-bit mantissas: 2.0 units of 2^-53, the rounding included):
 //
 //   angle reduction  |x| / 2 pi modulo 1 as the product of x's 53-bit
 //                    mantissa and the window of the bits of 1/(2 pi) that its
-//                    exponent selects (M. H. Payne, R. N. Hanek, 1983)
-//   sine, cosine     the fraction of a quarter turn in radians, split as
-//                    a_j + d with a_j = j 2^-8; (cos a_j, sin a_j) from a
+//                    exponent selects (M. H. Payne, R. N. Hanek, 1983), to 96
+//                    bits, folded to an eighth of a turn
+//   sine, cosine     of a_j + d, a_j = j pi/4096: (cos a_j, sin a_j) from a
 //                    table, turned by d in three shears (x -= t y, y += s x,
 //                    x -= t y with t = tan(d/2), s = sin d; A. W. Paeth,
 //                    1986), t and s by their Taylor polynomials
@@ -36,6 +37,7 @@
 
 namespace sdeb {
 
+// (cos, sin)(j pi/4096) in Q63 and Q64, j = 0 .. 1023 (an eighth of a turn).
 __device__ __forceinline__ ulonglong2 fixed_trig_table(uint32_t j) {
     return __ldg(reinterpret_cast<const ulonglong2 *>(kFixedTrig) + j);
 }
@@ -57,13 +59,25 @@ __device__ __forceinline__ int64_t with_sign(uint64_t v, uint32_t sign) {
     return ((int64_t)v ^ m) - m;
 }
 
-// (a b) >> 64, too small by at most 3, for a, b <= 2^63: the low product is
-// left out and the two cross products add without a carry.  Three wide
-// multiply-adds.
+// (a b) >> 64, too small by at most 3: the low product is left out and the two
+// cross products add without a carry, so a's and b's high words may take 32
+// bits between them less than their number (a, b <= 2^63, or a < 2^62 and any
+// b < 2^63.5).  Three wide multiply-adds.
 __device__ __forceinline__ uint64_t mul_top(uint64_t a, uint64_t b) {
     const uint32_t al = (uint32_t)a, ah = hi32(a), bl = (uint32_t)b, bh = hi32(b);
     const uint64_t cross = (uint64_t)al * bh + (uint64_t)ah * bl;
     return (uint64_t)ah * bh + hi32(cross);
+}
+
+// The position of the leading bit of h > 0, from the exponent of a truncating
+// float conversion (64 a clock; a count of leading zeros runs at 16).
+__device__ __forceinline__ int leading_bit(uint32_t h) { return (int)(__float_as_uint(__uint2float_rz(h)) >> 23) - 127; }
+
+// m 2^-q as a double, rounded to nearest (ties up), for m in [2^62, 2^63];
+// `sign` (0 or 1 << 31) its sign bit.
+__device__ __forceinline__ double normal_to_double(uint64_t m, int q, uint32_t sign) {
+    const uint64_t mant = (m + 512u) >> 10;  // 53 bits; their leading 1 adds 1 to the exponent field
+    return __hiloint2double((int)(sign + ((uint32_t)(1084 - q) << 20) + hi32(mant)), (int)(uint32_t)mant);
 }
 
 // v 2^-q as a double, rounded to nearest (ties up), `sign` (0 or 1 << 31) its
@@ -80,83 +94,129 @@ __device__ __forceinline__ double fixed_to_double(uint64_t v, int q, uint32_t si
     return __hiloint2double((int)((sign | (e << 20)) + hi32(mant)), (int)(uint32_t)mant);
 }
 
-// cos and sin (Q62) of f quarter turns, f in Q63 (< 2^63): rho = f pi/2 in
-// Q61, j = rho's multiple of 2^-8, d the rest (Q64).
-__device__ __forceinline__ void sincos_quarter(uint64_t f, uint64_t &c, uint64_t &s) {
-    const uint64_t rho = mul_top(f, 0x6487ED5110B4611AULL);  // pi/2 in Q62
-    const uint32_t j = (uint32_t)(rho >> 53);
-    const uint64_t d = (rho << 3) & 0x00FFFFFFFFFFFFFFULL;
-    // d 2^39, rounded, kept below 2^31 (d just under a table step rounds up to it, and z would be 2^32)
-    const uint32_t dh = min((uint32_t)((d + 0x1000000u) >> 25), 0x7FFFFFFFu);
-    const uint32_t z = (uint32_t)(((uint64_t)dh * dh) >> 30);       // d^2 2^48 (< 2^32: d < 2^-8)
-    const uint32_t a = __umulhi(z, 0xAAAAAAABu);                    // d^2/6 2^50
-    const uint32_t b = __umulhi(__umulhi(a, z), 0x0CCCCCCDu) >> 16;  // d^4/120 2^50
-    // sin d = d - d (d^2/6 - d^4/120); tan(d/2) = d/2 + d/2 (d^2/12 + d^4/120)
-    const uint64_t sn = d - (((uint64_t)dh * (a - b)) >> 25);
-    const uint64_t tn = (d >> 1) + (((uint64_t)dh * (a + 2 * b)) >> 27);
+// Cosine and sine of an angle of a quadrant, with their distance from an axis
+// folded to an eighth of a turn: `c` (Q63, at least 0.7) is the larger one,
+// `s` (Q64) the smaller one, `m` 2^-q the smaller one with its leading bit at
+// 62 and 62 bits of its own; swap: the sine is the larger one.
+struct Octant {
+    uint64_t c, s, m;
+    int q;
+    bool swap;
+    bool tiny;  // the smaller one is below 2^-15: m has lost bits, take the general functions
+};
+
+// turn (Q64) and turn_lo (its next 32 bits): the angle as a fraction of a turn.
+// d is exact to 2^-70, so the smaller one keeps its 54 bits from 2^-15 on, and
+// comes from the table's S_j (up to 2^-65 off) only where that is above 2^-10.4.
+__device__ __forceinline__ Octant sincos_octant(uint64_t turn, uint32_t turn_lo) {
+    Octant o;
+    uint64_t f = (turn << 2) | (turn_lo >> 30);  // quarter turns, Q64
+    uint32_t f_lo = turn_lo << 2;
+    const uint32_t fold = (uint32_t)((int32_t)hi32(f) >> 31);
+    f ^= ((uint64_t)fold << 32) | fold;  // f' = 1 - f
+    f_lo ^= fold;
+    o.swap = (((hi32(turn) >> 30) ^ fold) & 1u) != 0;  // quadrants 1 and 3: (cos, sin)(a + pi/2) = (-sin a, cos a)
+    const uint32_t j = hi32(f) >> 21;
+    const uint64_t rest = ((f << 10) | (f_lo >> 22)) & 0x7FFFFFFFFFFFFFFFULL;  // Q74, below 2^-11
+    const uint64_t d = mul_top(rest, 0x6487ED5110B4611AULL);                  // times pi/2 (Q62): Q72, below 2^-10.3
+    const uint32_t dh = (uint32_t)((d + 0x20000000u) >> 30);                  // Q42, below 2^31.7
+    const uint32_t z = hi32((uint64_t)dh * dh + 0x80000000u);                 // d^2, Q52
+    const uint32_t a = hi32((uint64_t)z * 0xAAAAAAABu + 0x80000000u);         // d^2/6, Q54
+    const uint32_t b = __umulhi(__umulhi(a, z), 0x0CCCCCCDu) >> 20;           // d^4/120, Q54
+    // sin d = d - d (d^2/6 - d^4/120), Q72; tan(d/2) = d/2 + d/2 (d^2/12 + d^4/120), Q63
+    const uint64_t sn = d - (((uint64_t)dh * (a - b)) >> 24);
+    const uint64_t tn = (d >> 10) + (((uint64_t)dh * (a + 2 * b)) >> 35);
     const ulonglong2 t = fixed_trig_table(j);
-    uint64_t x = t.x, y = t.y;
+    uint64_t x = t.x - mul_top(tn, t.y);
+    const uint64_t y = t.y + (mul_top(sn, x) >> 7);
     x -= mul_top(tn, y);
-    y += mul_top(sn, x);
-    x -= mul_top(tn, y);
-    c = x;
-    s = y;
+    o.c = x;
+    o.s = y;
+    const uint64_t own = j == 0 ? sn : y;  // S_0 = 0: the sine is sn itself, at its full resolution
+    const int up = 31 - leading_bit(hi32(own) | 1u);
+    o.m = (own << up) >> 1;
+    o.q = (j == 0 ? 71 : 63) + up;
+    o.tiny = j == 0 && hi32(own) < 0x02000000u;
+    return o;
 }
 
-// cos and sin of `turn` (Q64 fraction of a full turn) as Q62 magnitudes and
-// sign bits (0 or 1 << 31).
-__device__ __forceinline__ void sincos_turn(uint64_t turn, uint64_t &c, uint32_t &c_sign, uint64_t &s,
-                                            uint32_t &s_sign) {
-    uint64_t cq, sq;
-    sincos_quarter((turn << 1) & 0x7FFFFFFFFFFFFFFFULL, cq, sq);
-    const uint32_t th = hi32(turn);
-    const bool odd = (th & 0x40000000u) != 0;  // quadrants 1 and 3: (cos, sin)(a + pi/2) = (-sin a, cos a)
-    c = odd ? sq : cq;
-    s = odd ? cq : sq;
-    c_sign = (th + 0x40000000u) & 0x80000000u;  // quadrants 1 and 2
-    s_sign = th & 0x80000000u;                  // quadrants 2 and 3
+// Signs (0 or 1 << 31) of the cosine and the sine of `turn`.
+__device__ __forceinline__ uint32_t cos_sign(uint64_t turn) { return (hi32(turn) + 0x40000000u) & 0x80000000u; }
+__device__ __forceinline__ uint32_t sin_sign(uint64_t turn) { return hi32(turn) & 0x80000000u; }
+
+// (cos, sin) of an octant's angle.
+__device__ __forceinline__ void octant_to_double(const Octant &o, uint32_t c_sign, uint32_t s_sign, double &c,
+                                                 double &s) {
+    const double large = normal_to_double(o.c, 63, o.swap ? s_sign : c_sign);
+    const double small = normal_to_double(o.m, o.q, o.swap ? c_sign : s_sign);
+    c = o.swap ? small : large;
+    s = o.swap ? large : small;
 }
 
-// Phases whose sine and cosine are taken here: 2^-11 <= |x| < 2^21.  Smaller
-// ones (whose sine would lose relative precision in fixed point), larger and
-// non-finite ones go to CUDA's sincos, out of line.
+// Phases whose sine and cosine are taken here, in line: 2^-11 <= |x| < 2^21.
+// Smaller ones are their own reduced angle (sincos_small); larger ones, and
+// those within 2^-15 of a multiple of a quarter turn, go out of line.
 constexpr uint32_t kPhaseMinHi = 0x3F400000u;                 // high word of 2^-11
 constexpr uint32_t kPhaseSpanHi = 0x41400000u - kPhaseMinHi;  // to 2^21
 
 __device__ __forceinline__ bool phase_fixed(uint32_t hi) { return (hi & 0x7fffffffu) - kPhaseMinHi < kPhaseSpanHi; }
+__device__ __forceinline__ bool phase_small(uint32_t hi) { return (hi & 0x7fffffffu) < kPhaseMinHi; }
 
-// |x| / (2 pi) modulo 1 in Q64 (hi, lo: the words of a phase in the range
-// above).  |x| = m 2^-s with s in [32, 63], so the fraction is m times the 96
-// bits of 1/(2 pi) from the one that weighs 2^(s - 64) on, modulo 2^64.  (Any
-// other phase gives some value.)
-__device__ __forceinline__ uint64_t turn_fraction(uint32_t hi, uint32_t lo) {
-    const uint32_t sh = 1043u - ((hi >> 20) & 0x7ffu);  // s - 32
-    const uint32_t w2 = __funnelshift_r(0x28BE60DBu, 0u, sh);
-    const uint32_t w1 = __funnelshift_r(0x9391054Au, 0x28BE60DBu, sh);
-    const uint32_t w0 = __funnelshift_r(0x7F09D5F4u, 0x9391054Au, sh);
+// |x| / (2 pi) modulo 1 in Q64 and the next 32 bits (hi, lo: the words of a
+// phase in the range above; BIG: of one from 2^21 to 2^53), less than 2^-74 too
+// small.  |x| = m 2^-s with s in [32, 63], so the fraction is m times the bits
+// of 1/(2 pi) from the one that weighs 2^(s - 64) on, modulo 2^64; BIG, s in
+// [0, 31], from one word further on.  (Any other phase gives some value.)
+template <bool BIG = false>
+__device__ __forceinline__ uint64_t turn_fraction(uint32_t hi, uint32_t lo, uint32_t &next) {
+    constexpr uint32_t kBits[5] = {0u, 0x28BE60DBu, 0x9391054Au, 0x7F09D5F4u, 0x7D4D3770u};
+    constexpr int o = BIG ? 1 : 0;
+    const uint32_t sh = 1043u - ((hi >> 20) & 0x7ffu);  // s - 32; a funnel shift takes it modulo 32
+    const uint32_t w2 = __funnelshift_r(kBits[o + 1], kBits[o], sh);
+    const uint32_t w1 = __funnelshift_r(kBits[o + 2], kBits[o + 1], sh);
+    const uint32_t w0 = __funnelshift_r(kBits[o + 3], kBits[o + 2], sh);
     const uint32_t m0 = lo, m1 = (hi & 0xfffffu) | 0x100000u;
-    uint64_t r = (uint64_t)m0 * w2 + __umulhi(m0, w1);
+    const uint64_t t = (uint64_t)m0 * w1 + __umulhi(m0, w0);
+    const uint64_t u = (uint64_t)m1 * w0 + (uint32_t)t;
+    uint64_t r = (uint64_t)m0 * w2 + hi32(t);
     r += (uint64_t)m1 * w1;
-    r += __umulhi(m1, w0);
-    return r + ((uint64_t)(m1 * w2) << 32);
+    r += hi32(u);
+    next = (uint32_t)u;
+    uint32_t top = m1 * w2;
+    if constexpr (BIG) top += m0 * __funnelshift_r(kBits[1], kBits[0], sh);  // whole turns but for m0's bits below them
+    return r + ((uint64_t)top << 32);
 }
 
+// (cos, sin) of |x| < 2^-11 by their Taylor polynomials (the terms left out
+// are below 2^-77 and 2^-75).
+__device__ __forceinline__ double2 sincos_small(double x) {
+    const double x2 = x * x;
+    return make_double2(fma(x2, fma(x2, 1.0 / 24.0, -0.5), 1.0), fma(x * x2, fma(x2, 1.0 / 120.0, -1.0 / 6.0), x));
+}
+
+// (cos, sin) of any phase: from 2^21 to 2^53 as in line, else by CUDA's sincos.
 static __device__ __noinline__ double2 sincos_general(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x);
     double2 r;
+    if ((hi & 0x7fffffffu) - (kPhaseMinHi + kPhaseSpanHi) < 0x43400000u - (kPhaseMinHi + kPhaseSpanHi)) {
+        uint32_t next;
+        const uint64_t turn = turn_fraction<true>(hi, (uint32_t)__double2loint(x), next);
+        const Octant o = sincos_octant(turn, next);
+        octant_to_double(o, cos_sign(turn), sin_sign(turn) ^ (hi & 0x80000000u), r.x, r.y);
+        if (!o.tiny) return r;
+    }
     sincos(x, &r.y, &r.x);
     return r;
 }
 
 __device__ __forceinline__ void sincos_fixed(double x, double &s, double &c) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    if (phase_fixed(hi)) {
-        uint64_t cv, sv;
-        uint32_t cs, ss;
-        sincos_turn(turn_fraction(hi, lo), cv, cs, sv, ss);
-        c = fixed_to_double(cv, 62, cs);
-        s = fixed_to_double(sv, 62, ss ^ (hi & 0x80000000u));
-    } else {
-        const double2 r = sincos_general(x);
+    uint32_t next;
+    const uint64_t turn = turn_fraction(hi, lo, next);
+    const Octant o = sincos_octant(turn, next);
+    octant_to_double(o, cos_sign(turn), sin_sign(turn) ^ (hi & 0x80000000u), c, s);
+    if (!phase_fixed(hi) || o.tiny) {
+        const double2 r = phase_small(hi) ? sincos_small(x) : sincos_general(x);
         c = r.x;
         s = r.y;
     }
@@ -208,16 +268,38 @@ __device__ __forceinline__ uint64_t normal_radius(uint32_t w, int &h) {
     return (r0 << 2) + (mul_top(r0, c << 23) >> 17);
 }
 
+static __device__ __noinline__ double2 cospi_sinpi_general(double x) {
+    double2 r;
+    sincospi(x, &r.y, &r.x);
+    return r;
+}
+
+// p 2^-q as a double for p in [2^60, 2^62]: a product of two numbers in
+// [2^62, 2^63].
+__device__ __forceinline__ double product_to_double(uint64_t p, int q, uint32_t sign) {
+    const int up = hi32(p) < 0x20000000u ? 2 : 1;
+    return normal_to_double(p << up, q + up, sign);
+}
+
 // Eq. 3 for the word pair (w_first, w_second): radius sqrt(-2 ln u1), angle u2
-// turns.
+// turns.  Angles within 2^-15 of a multiple of a quarter turn take the product
+// of the rounded radius and CUDA's sincospi.
 __device__ __forceinline__ void box_muller_fixed(uint32_t w_first, uint32_t w_second, double &n_cos, double &n_sin) {
     int h;
     const uint64_t r = normal_radius(w_first, h);
-    uint64_t cv, sv;
-    uint32_t cs, ss;
-    sincos_turn(((uint64_t)w_second << 32) | 0x80000000u, cv, cs, sv, ss);
-    n_cos = fixed_to_double(mul_top(r, cv), 61 - h, cs);
-    n_sin = fixed_to_double(mul_top(r, sv), 61 - h, ss);
+    const uint64_t turn = ((uint64_t)w_second << 32) | 0x80000000u;
+    const Octant o = sincos_octant(turn, 0);
+    const uint32_t cs = cos_sign(turn), ss = sin_sign(turn);
+    const double large = product_to_double(mul_top(r, o.c), 62 - h, o.swap ? ss : cs);
+    const double small = product_to_double(mul_top(r, o.m), o.q - 1 - h, o.swap ? cs : ss);
+    n_cos = o.swap ? small : large;
+    n_sin = o.swap ? large : small;
+    if (o.tiny) {
+        const double2 t = cospi_sinpi_general(__uint2double_rn(w_second) * 0x1p-31 + 0x1p-32);
+        const double radius = normal_to_double(r, 63 - h, 0u);
+        n_cos = radius * t.x;
+        n_sin = radius * t.y;
+    }
 }
 
 }  // namespace sdeb
