@@ -84,18 +84,18 @@ def _pi_bits():
     return 16 * atan_inv(5) - 4 * atan_inv(239)
 
 
-def fixed_tables(step=(1, 256), rows=403, q_cos=62, q_sin=62, q_log=58, up=2):
-    """(cos, sin)(j step) in Q(q_cos) and Q(q_sin), j < rows, the cosines `up` units up (of use where rows pass
+def fixed_tables(step=(1, 256), rows=403, q_cos=62, q_sin=62, q_log=58, up=(2, 0)):
+    """(cos, sin)(j step) in Q(q_cos) and Q(q_sin), j < rows, the cosines up[0] units up (of use where rows pass
     pi/2: a rotation's rounding then leaves none below 0), and (ln c, c), c in Q15 the largest with m c <= 1 for
-    every m below (257 + j) / 512, ln c in Q(q_log)."""
+    every m below (257 + j) / 512, ln c in Q(q_log), up[1] units up."""
     trig = []
     for j in range(rows):
         c, s = _sincos_bits(j * step[0], step[1])
-        trig.append((_rounded(c, q_cos) + up, _rounded(s, q_sin)))
+        trig.append((_rounded(c, q_cos) + up[0], _rounded(s, q_sin)))
     log = []
     for j in range(256):
         c = (512 << 15) // (257 + j)
-        log.append((_rounded(_ln_bits(c, 1 << 15), q_log), c))
+        log.append((_rounded(_ln_bits(c, 1 << 15), q_log) + up[1], c))
     return trig, log
 
 
@@ -111,7 +111,7 @@ def _write_if_changed(path, content):
 
 def generate_fixed_tables():
     parts = ["// Generated by build.py: tables of fixed_math.cuh.\n#pragma once\nnamespace sdeb {\n"]
-    tables = fixed_tables((_pi_bits(), 4096 << _BITS), 1024, 63, 64, 58, 0)
+    tables = fixed_tables((_pi_bits(), 4096 << _BITS), 1024, 63, 64, 64, (0, 2))
     for name, rows in zip(("kFixedTrig", "kFixedLog"), tables):
         parts.append("static __device__ const __align__(16) unsigned long long %s[%d][2] = {\n" % (name, len(rows)))
         parts += ["{0x%016xull, 0x%016xull},\n" % row for row in rows]

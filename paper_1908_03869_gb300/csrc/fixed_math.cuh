@@ -6,9 +6,10 @@
 // integer adds or shifts.  CUDA's double sincos, log and sqrt are sequences
 // on that one pipe: they were 59 of the 65.6 FP64 instructions per
 // oscillator-step of the Kuramoto kernel.  Here they are integer sequences,
-// each result rounded to double once; a sine or cosine is within 2^-52 of the
-// exact one relative to itself, however small it is (measured on the host
-// against 64-bit mantissas: 2.0 units of 2^-53, the rounding included):
+// each result rounded to double once and right relative to itself, however
+// small it is (the largest errors on the host against 64-bit mantissas, in
+// units of 2^-53: sine and cosine 2.0, the radius before its rounding 0.3,
+// normals 2.0, 2.8 next to a multiple of a quarter turn):
 //
 //   angle reduction  |x| / 2 pi modulo 1 as the product of x's 53-bit
 //                    mantissa and the window of the bits of 1/(2 pi) that its
@@ -43,7 +44,7 @@ __device__ __forceinline__ ulonglong2 fixed_trig_table(uint32_t j) {
 }
 
 struct FixedLogEntry {
-    uint64_t lnc;  // ln c in Q58
+    uint64_t lnc;  // ln c in Q64, 2 units up (the bits that normal_radius shifts out then round)
     uint32_t c;    // Q15
 };
 __device__ __forceinline__ FixedLogEntry fixed_log_table(uint32_t j) {
@@ -234,7 +235,8 @@ __device__ __forceinline__ uint64_t normal_radius(uint32_t w, int &h) {
     // u = m 2^-n, m in [1/2, 1) in Q64
     const int n = __clz((int)w);
     const uint64_t m = (((uint64_t)w << 32) | 0x80000000u) << n;
-    const FixedLogEntry t = fixed_log_table((hi32(m) >> 23) & 255u);
+    const uint32_t j = (hi32(m) >> 23) & 255u;
+    const FixedLogEntry t = fixed_log_table(j);
     // r = 1 - m c: m has 33 leading bits at most, c is in Q15, so r is exact
     // in Q48 and below 2^-7.9
     const uint64_t r48 = (1ULL << 48) - ((uint64_t)hi32(m) * (2u * t.c) + ((uint32_t)m != 0 ? t.c : 0u));
@@ -247,16 +249,27 @@ __device__ __forceinline__ uint64_t normal_radius(uint32_t w, int &h) {
     uint64_t q = 0x2AAAAAAAAAAAAAABULL + (((uint64_t)rr * i) >> 9);  // Q63
     q = (1ULL << 62) + (mul_top(r, q) >> 6);                       // Q63
     q = (1ULL << 62) + (mul_top(r, q) >> 7);                       // Q62
-    const uint64_t p = mul_top(r, q);                              // Q68
-    const uint64_t base = (uint64_t)(uint32_t)n * 0x02C5C85FDF473DE7ULL + t.lnc;  // n ln 2 + ln c in Q58
-    // u within 2^-9 of 1: the series alone, kept at its full resolution
-    const uint64_t v = base == 0 ? p : base + (p >> 10);
-    const int ex = base == 0 ? 68 : 58;
+    // -ln u = n ln 2 + ln c - ln(1 - r): in Q58, for u past 1/2 in Q62; for u
+    // past 1 - 2^-9, where ln c = 0, as r (Q70) times q below
+    const bool near_one = n == 0 && j == 255u;
+    uint64_t v = r;
+    int ex = 70;
+    if (!near_one) {
+        const uint64_t frac = t.lnc + (mul_top(r, q) >> 4);  // Q64
+        v = (uint64_t)(uint32_t)n * 0x02C5C85FDF473DE7ULL + (frac >> (n == 0 ? 2 : 6));
+        ex = n == 0 ? 62 : 58;
+    }
     // 2 L = a 2^(64 - ex - up), a = A 2^-63 in [1/4, 1), up even
-    const int top = (int)(__float_as_uint(__uint2float_rz(hi32(v))) >> 23) - 127;
-    const int up = (30 - top) & ~1;
-    const uint64_t A = v << up;
+    const int up = (30 - leading_bit(hi32(v))) & ~1;
+    uint64_t A = v << up;
     h = (64 - ex - up) >> 1;
+    if (near_one) {
+        A = mul_top(A, q) << 2;
+        if ((A >> 63) != 0) {
+            A >>= 2;
+            ++h;
+        }
+    }
     // y below 1/sqrt(a) by 2^-23 to 2^-20.7 (so e > 0): the seed's 2^-22.9 and
     // three float roundings against a bias of 2^-21.4
     const float y0 = rsqrt_seed_f32(__uint2float_rn(hi32(A)) * 0x1p-31f);

@@ -5,7 +5,9 @@ relative to each result, however small it is, in units of 2^-53.
 Bounds: the rounding to double is 1 unit at most (half a unit in the last
 place next to a power of two); the sine's polynomial is off by 1.1 units at
 most (its d^2/6 is kept to 2^-55 and d^2 to 2^-52.4), so 2.25 for sine and
-cosine.
+cosine; the radius has half a unit before it is rounded, a normal is the
+product of the two with one rounding, or, near a multiple of a quarter turn, of
+three rounded factors: 3.
 """
 import os
 import re
@@ -67,6 +69,13 @@ static long double units(double got, long double want) { return want == 0 ? (got
 static std::mt19937_64 g(11);
 static double uniform(double a, double b) { return std::uniform_real_distribution<double>(a, b)(g); }
 static double sign() { return g() & 1 ? 1.0 : -1.0; }
+static long double log_of(uint32_t w) {  // ln((w + 1/2) 2^-32)
+    return w >> 31 ? log1pl(-((0xffffffffu - w) + 0.5L) * 0x1p-32L) : logl((w + 0.5L) * 0x1p-32L);
+}
+static uint32_t word(int kind, long i) {
+    const uint32_t d = (uint32_t)std::exp2(uniform(0, 32));
+    return kind == 0 ? (uint32_t)g() : kind == 1 ? d - 1 : kind == 2 ? 0xffffffffu - (d - 1) : kind == 3 ? (uint32_t)i : 0xffffffffu - (uint32_t)i;
+}
 int main(int, char **argv) {
     const std::string what = argv[1];
     long double worst = 0;
@@ -89,6 +98,33 @@ int main(int, char **argv) {
                 sincos_fixed(x, s, c);
                 see(units(s, sinl(x)));
                 see(units(c, cosl(x)));
+            }
+    } else if (what == "radius") {
+        for (int seed = -1; seed <= 1; ++seed) {
+            g_seed_error = seed * 0x1.125p-23;
+            for (int kind = 0; kind < 5; ++kind)
+                for (long i = 0; i < 200000; ++i) {
+                    const uint32_t w = word(kind, i);
+                    int h;
+                    const uint64_t r = normal_radius(w, h);
+                    const long double want = sqrtl(-2 * log_of(w));
+                    see(fabsl((ldexpl((long double)r, h - 63) - want) / want) * 0x1p53L);
+                }
+        }
+    } else if (what == "normals") {
+        for (int kind = 0; kind < 5; ++kind)
+            for (long i = 0; i < 300000; ++i) {
+                const uint32_t a = word(kind % 3, i);
+                const uint32_t b = kind < 3 ? (uint32_t)g() : (uint32_t)((g() << 30) + (int64_t)(sign() * std::exp2(uniform(0, 30))));
+                double z[2];
+                box_muller_fixed(a, b, z[0], z[1]);
+                const uint64_t t = 2ull * b + 1;  // 33 bits of a turn
+                const long double r = sqrtl(-2 * log_of(a)), f = (t & 0x7fffffffu) * 0x1p-31L;
+                long double s = f <= 0.5L ? sinl(M_PI_2l * f) : cosl(M_PI_2l * (1 - f));
+                long double c = f <= 0.5L ? cosl(M_PI_2l * f) : sinl(M_PI_2l * (1 - f));
+                const int q = (int)(t >> 31);
+                see(units(z[0], r * (q == 0 ? c : q == 1 ? -s : q == 2 ? -c : s)));
+                see(units(z[1], r * (q == 0 ? s : q == 1 ? c : q == 2 ? -s : -c)));
             }
     }
     printf("%.4Lf\n", worst);
@@ -126,6 +162,6 @@ def worst(program):
     return lambda what: float(run(what))
 
 
-@pytest.mark.parametrize("what,bound", [("phases", 2.25)])
+@pytest.mark.parametrize("what,bound", [("phases", 2.25), ("radius", 0.5), ("normals", 3.0)])
 def test_errors_relative_to_the_result(worst, what, bound):
     assert worst(what) <= bound
