@@ -66,9 +66,12 @@ __device__ __forceinline__ void store_units(Real *row, int units, int u0, const 
 
 // Coupling-sum reducers.  WarpGroupSum<G>: butterfly over the G lanes of an
 // orbit inside one warp, in the given type or, for models with fixed-point
-// sums (FP64 phases), in 64-bit integers: exact, so the totals are the same
-// bits for every layout.  `bad` becomes true in every lane of an orbit that
-// has a lane with a non-finite phase.
+// sums (FP64 phases), as FixedSums: exact, so the totals are the same bits for
+// every layout.  `fixed` adds an orbit's sums and joins its lanes' `seen` (mine:
+// the lane has units), and says whether some orbit of the warp lacks a bit or
+// has a bad one; LIKELY: lanes usually have both bits by themselves.
+// `largest` takes a maximum, `any` is true where it is for some orbit of the
+// warp.
 template <int G>
 struct WarpGroupSum {
     static constexpr bool kFixedSums = true;
@@ -77,16 +80,53 @@ struct WarpGroupSum {
 #pragma unroll
         for (int q = 0; q < NR; ++q) r[q] = group_sum<G>(r[q]);
     }
-    __device__ __forceinline__ void fixed(int64_t (&r)[2], bool &bad) const {
+    template <bool LIKELY>
+    __device__ __forceinline__ bool fixed(FixedSums &t, bool mine) const {
+        bool special = t.seen != FixedSums::kAllSeen;
+        if constexpr (G > 1) {
+            // the votes ahead of the shuffles, which hide them
+            if (!LIKELY || !__all_sync(0xffffffffu, !special || !mine)) {
+                const unsigned group = (0xffffffffu >> (32 - G)) << (threadIdx.x & 31 & ~(G - 1));
+                uint32_t joined = 0;
+#pragma unroll
+                for (uint32_t bit = 1; bit < 8; bit <<= 1)
+                    if ((__ballot_sync(0xffffffffu, (t.seen & bit) != 0) & group) != 0) joined |= bit;
+                t.seen = joined;
+                special = __any_sync(0xffffffffu, joined != FixedSums::kAllSeen);
+            } else {
+                t.seen = FixedSums::kAllSeen;
+                special = false;
+            }
+        }
 #pragma unroll
         for (int off = 1; off < G; off <<= 1) {
-            r[0] += __shfl_xor_sync(0xffffffffu, (long long)r[0], off);
-            r[1] += __shfl_xor_sync(0xffffffffu, (long long)r[1], off);
+            t.top[0] += __shfl_xor_sync(0xffffffffu, (long long)t.top[0], off);
+            t.top[1] += __shfl_xor_sync(0xffffffffu, (long long)t.top[1], off);
+            t.low += __shfl_xor_sync(0xffffffffu, t.low, off);
         }
-        if constexpr (G > 1) {
-            const unsigned all = __ballot_sync(0xffffffffu, bad);
-            bad = ((all >> (threadIdx.x & 31 & ~(G - 1))) & (0xffffffffu >> (32 - G))) != 0;
+        return special;
+    }
+    // The two sums as doubles; SHARE: one on every second lane, then exchanged.
+    template <bool SHARE>
+    __device__ __forceinline__ void values(const FixedSums &t, double (&red)[2]) const {
+        if constexpr (SHARE && G > 1) {
+            const bool odd = (threadIdx.x & 1u) != 0;
+            const double mine = t.value<true>(odd ? 1 : 0), other = __shfl_xor_sync(0xffffffffu, mine, 1);
+            red[0] = odd ? other : mine;
+            red[1] = odd ? mine : other;
+        } else {
+            red[0] = t.value<SHARE>(0);
+            red[1] = t.value<SHARE>(1);
         }
+    }
+    __device__ __forceinline__ uint32_t largest(uint32_t v) const {
+#pragma unroll
+        for (int off = 1; off < G; off <<= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, off));
+        return v;
+    }
+    __device__ __forceinline__ bool any(bool b) const {
+        if constexpr (G > 1) return __any_sync(0xffffffffu, b);
+        else return b;
     }
 };
 
@@ -94,32 +134,50 @@ struct WarpGroupSum {
 // fixed-point sums: warp butterflies, then the warps' partials exchanged
 // through shared memory (double-buffered, one barrier a call: the block's, or
 // named barrier BAR where the block has other warps).
+struct TeamPartial {
+    longlong2 sum;
+    uint2 word;
+};
+
 template <int NW, int BAR = 0>
 struct TeamFixedSum {
     static constexpr bool kFixedSums = true;
-    longlong2 *buf;  // shared memory, [2][NW]
-    int *bad_buf;    // shared memory, [2][NW]
+    TeamPartial *buf;  // shared memory, [2][NW]
     int flip;
-    __device__ __forceinline__ void fixed(int64_t (&r)[2], bool &bad) {
-        WarpGroupSum<32>().fixed(r, bad);
-        const int warp = threadIdx.x >> 5;
-        if ((threadIdx.x & 31) == 0) {
-            buf[flip * NW + warp] = make_longlong2(r[0], r[1]);
-            bad_buf[flip * NW + warp] = bad;
-        }
+    __device__ __forceinline__ const TeamPartial *exchange(const TeamPartial &mine) {
+        if ((threadIdx.x & 31) == 0) buf[flip * NW + (threadIdx.x >> 5)] = mine;
         if constexpr (BAR == 0) __syncthreads();
         else asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NW * 32) : "memory");
-        r[0] = r[1] = 0;
-        bad = false;
+        const TeamPartial *all = buf + flip * NW;
+        flip ^= 1;
+        return all;
+    }
+    template <bool LIKELY>
+    __device__ __forceinline__ bool fixed(FixedSums &t, bool mine) {
+        (void)WarpGroupSum<32>().fixed<LIKELY>(t, mine);
+        const TeamPartial *all = exchange({make_longlong2(t.top[0], t.top[1]), make_uint2(t.low, t.seen)});
+        t = FixedSums();
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
-            const longlong2 t = buf[flip * NW + w];
-            r[0] += t.x;
-            r[1] += t.y;
-            bad = bad || bad_buf[flip * NW + w] != 0;
+            t.top[0] += all[w].sum.x;
+            t.top[1] += all[w].sum.y;
+            t.low += all[w].word.x;
+            t.seen |= all[w].word.y;
         }
-        flip ^= 1;
+        return t.seen != FixedSums::kAllSeen;
     }
+    template <bool SHARE>
+    __device__ __forceinline__ void values(const FixedSums &t, double (&red)[2]) const {
+        WarpGroupSum<32>().values<SHARE>(t, red);
+    }
+    __device__ __forceinline__ uint32_t largest(uint32_t v) {
+        v = WarpGroupSum<32>().largest(v);
+        const TeamPartial *all = exchange({make_longlong2(0, 0), make_uint2(v, 0)});
+#pragma unroll
+        for (int w = 0; w < NW; ++w) v = max(v, all[w].word.x);
+        return v;
+    }
+    __device__ __forceinline__ bool any(bool b) const { return b; }  // the same orbit in every warp
 };
 
 // Whether model M's coupling sums go through reducer RED in fixed point.
@@ -476,9 +534,8 @@ __device__ __forceinline__ void em_forward_body(const ForwardArgs &a) {
     // an orbit on more than a warp has the thread block to itself
     std::conditional_t<(G > 32), TeamFixedSum<(G + 31) / 32>, WarpGroupSum<(G > 32 ? 32 : G)>> reduce;
     if constexpr (G > 32) {
-        __shared__ longlong2 team_sums[2 * (G / 32)];
-        __shared__ int team_bad[2 * (G / 32)];
-        reduce = {team_sums, team_bad, 0};
+        __shared__ TeamPartial team[2 * (G / 32)];
+        reduce = {team, 0};
     }
     const NoiseLane<P> noise(gorb, u0, a.keys);
     // Steps run in runs that end at the next frame, checkpoint or k_end (and,

@@ -31,6 +31,40 @@
 
 namespace sdeb {
 
+// Two sums of terms of magnitude at most 1 as exact integers in Q60: the upper
+// bits in Q54 (of at most 256 terms: 2^62), the last 6 bits in the 16-bit halves
+// of `low`.
+struct FixedSums {
+    static constexpr int kUnits = 4;             // terms added up before they are split: 2^62
+    static constexpr uint32_t kLarge = 1u << 22;  // high word of 2^-6 in Q60
+    // of `seen`: a non-finite phase; sum q has a term of at least 2^-6: kSeen << q
+    static constexpr uint32_t kBad = 1u, kSeen = 2u, kAllSeen = 6u;
+    int64_t top[2] = {0, 0};
+    uint32_t low = 0, seen = 0;
+
+    __device__ __forceinline__ void take(int64_t (&part)[2]) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            top[q] += part[q] >> 6;
+            low += ((uint32_t)part[q] & 63u) << (16 * q);
+            part[q] = 0;
+        }
+    }
+    __device__ __forceinline__ void take_unit(double2 r, uint32_t (&large)[2]) {
+        const uint32_t hc = (uint32_t)__double2hiint(r.x), hs = (uint32_t)__double2hiint(r.y);
+        const uint64_t c = to_q60(hc, (uint32_t)__double2loint(r.x)), s = to_q60(hs, (uint32_t)__double2loint(r.y));
+        int64_t part[2] = {with_sign(c, hc & 0x80000000u), with_sign(s, hs & 0x80000000u)};
+        large[0] |= hi32(c);
+        large[1] |= hi32(s);
+        take(part);
+    }
+    template <bool JUMP>
+    __device__ __forceinline__ double value(int q) const {
+        const uint32_t l = low >> (16 * q) & 0xffffu;
+        return sum_to_double<JUMP>((q != 0 ? top[1] : top[0]) + (l >> 6), l << 26, 54);
+    }
+};
+
 // Kuramoto, Eq. 5/6, drift in its mean-field form: with C = sum_j cos x_j and
 // S = sum_j sin x_j, sum_j sin(x_j - x_i) = S cos x_i - C sin x_i.
 // PAPER = false: p = (K, sigma, omega_1..omega_n); true: p = (K, omega, p_1..p_n).
@@ -111,17 +145,19 @@ struct KuramotoLane {
     }
 
     // FP64: sines, cosines and the orbit's sums over the lanes of `reduce`, the
-    // sums as integers in Q54 (at most 256 units: below 2^62; a term's dropped
-    // bits are below 2^-54 of full scale, what an FP64 sum past 1/2 rounds by).
+    // sums as exact integers in Q60, so that every layout gets the same bits
+    // (FixedSums).  A term is off by 2^-60 at most, which is below what an FP64
+    // sum rounds by unless all the orbit's terms are small; small_sum then takes
+    // the sum again at their scale.
     // All units go through the fixed-point sequences, in one straight block
-    // with the step's noise for the scheduler; a unit whose phase is outside
-    // their range (its values there mean nothing) is then taken again.
+    // with the step's noise for the scheduler; the units outside their range
+    // (whose values there mean nothing) are then taken again.
     template <class RED>
     __device__ __forceinline__ void fixed_sums(const double (&z)[P], int u0, int units, RED &reduce,
                                                double (&red)[NR]) {
-        int64_t sum[2] = {0, 0};
-        bool bad = false;
-        uint32_t again = 0;
+        FixedSums t;
+        uint32_t again = 0, large[NR] = {0, 0};
+        int64_t part[NR] = {0, 0};
 #pragma unroll
         for (int i = 0; i < P; ++i) {
             const uint32_t hi = (uint32_t)__double2hiint(z[i]);
@@ -132,9 +168,13 @@ struct KuramotoLane {
             octant_to_double(o, c_sign, s_sign, cs[i], sn[i]);
             const bool in_range = phase_fixed(hi) && !o.tiny, mine = u0 + i < units;
             again |= mine && !in_range ? 1u << i : 0u;
-            const uint64_t keep = mine && in_range ? ~0ULL : 0ULL, lg = o.c >> 9, sm = o.s >> 10;
-            sum[0] += with_sign((o.swap ? sm : lg) & keep, c_sign);
-            sum[1] += with_sign((o.swap ? lg : sm) & keep, s_sign);
+            const uint64_t keep = mine && in_range ? ~0ULL : 0ULL, lg = o.c >> 3, sm = o.s >> 4;
+            const uint64_t c = (o.swap ? sm : lg) & keep, s = (o.swap ? lg : sm) & keep;
+            part[0] += with_sign(c, c_sign);
+            part[1] += with_sign(s, s_sign);
+            large[0] |= hi32(c);
+            large[1] |= hi32(s);
+            if (i % FixedSums::kUnits == FixedSums::kUnits - 1 || i == P - 1) t.take(part);
         }
         // rolled: the instruction cache holds little more than the block above
 #pragma unroll 1
@@ -149,20 +189,50 @@ struct KuramotoLane {
                 cs[j] = j == i ? r.x : cs[j];
                 sn[j] = j == i ? r.y : sn[j];
             }
-            if (isfinite(zi)) {
-                sum[0] += __double2ll_rn(r.x * 0x1p54);
-                sum[1] += __double2ll_rn(r.y * 0x1p54);
-            } else {
-                bad = true;
-            }
+            if (isfinite(zi)) t.take_unit(r, large);
+            else t.seen |= FixedSums::kBad;
         }
-        reduce.fixed(sum, bad);
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const uint32_t sign = hi32((uint64_t)sum[q]) & 0x80000000u;
-            red[q] = fixed_to_double((uint64_t)with_sign((uint64_t)sum[q], sign), 54, sign);
-            if (bad) red[q] = __longlong_as_double(0x7ff8000000000000LL);
+        for (int q = 0; q < NR; ++q) t.seen |= large[q] >= FixedSums::kLarge ? FixedSums::kSeen << q : 0u;
+        const bool some_small = reduce.template fixed<(P >= 4)>(t, u0 < units);
+        reduce.template values<(P >= 4)>(t, red);
+        if (some_small) {
+#pragma unroll 1
+            for (int q = 0; q < NR; ++q) {
+                const bool own = (t.seen & FixedSums::kSeen << q) == 0;
+                if (!reduce.any(own)) continue;
+                double v[P];
+#pragma unroll
+                for (int i = 0; i < P; ++i) v[i] = q == 0 ? cs[i] : sn[i];
+                const double sum = small_sum(v, u0, units, reduce);
+                red[0] = own && q == 0 ? sum : red[0];
+                red[1] = own && q == 1 ? sum : red[1];
+            }
+            if ((t.seen & FixedSums::kBad) != 0) red[0] = red[1] = __longlong_as_double(0x7ff8000000000000LL);
         }
+    }
+
+    // The sum of an orbit's terms v, again as an exact integer: of the terms
+    // times the power of two that takes their largest to 62 bits less
+    // log2(units).  (The warp's other orbits come along.)
+    template <class RED>
+    static __device__ __forceinline__ double small_sum(const double (&v)[P], int u0, int units, RED &reduce) {
+        uint32_t top = 1u << 20;  // high word of the largest term, or of the least normal number
+#pragma unroll
+        for (int i = 0; i < P; ++i)
+            if (u0 + i < units) top = max(top, (uint32_t)__double2hiint(v[i]) & 0x7fffffffu);
+        const int e_top = (int)(reduce.largest(top) >> 20);  // terms are below 2^(e_top - 1022)
+        const int q = 30 + __clz(units - 1);
+        FixedSums t;
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            const uint32_t hi = (uint32_t)__double2hiint(v[i]);
+            const int e = (int)(hi >> 20 & 0x7ffu);
+            const uint64_t m = ((uint64_t)((hi & 0xfffffu) | (e != 0 ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(v[i]);
+            if (u0 + i < units) t.top[0] += with_sign(m << (q - 53) >> min(e_top - max(e, 1), 63), hi & 0x80000000u);
+        }
+        (void)reduce.template fixed<false>(t, true);
+        return sum_to_double<true>(t.top[0], 0u, q) * __hiloint2double((e_top + 1) << 20, 0);
     }
 
     // f dt = (K/n) dt (S cos x_i - C sin x_i) + omega_i dt, with (K/n) dt S

@@ -135,9 +135,8 @@ __global__ void __launch_bounds__(SplitShape<G, P>::kThreads) em_split_kernel(co
         if constexpr (kKahan) {
             return EightsSum<M, G, P>{model};
         } else if constexpr (G > 32) {
-            __shared__ longlong2 team_sums[2 * (G / 32)];
-            __shared__ int team_bad[2 * (G / 32)];
-            return TeamFixedSum<Shape::kConsumerWarps, 1>{team_sums, team_bad, 0};
+            __shared__ TeamPartial team[2 * (G / 32)];
+            return TeamFixedSum<Shape::kConsumerWarps, 1>{team, 0};
         } else {
             return WarpGroupSum<G>();
         }

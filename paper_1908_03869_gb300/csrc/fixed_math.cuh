@@ -81,18 +81,47 @@ __device__ __forceinline__ double normal_to_double(uint64_t m, int q, uint32_t s
     return __hiloint2double((int)(sign + ((uint32_t)(1084 - q) << 20) + hi32(mant)), (int)(uint32_t)mant);
 }
 
-// v 2^-q as a double, rounded to nearest (ties up), `sign` (0 or 1 << 31) its
-// sign bit.  v = 0 gives a magnitude below 2^-100.  The shift comes from the
-// exponent of a truncating float conversion (64 a clock; a count of leading
-// zeros runs at 16).
-__device__ __forceinline__ double fixed_to_double(uint64_t v, int q, uint32_t sign) {
-    const bool low = hi32(v) == 0;
-    const uint32_t h = low ? (uint32_t)v : hi32(v), l = low ? 0u : (uint32_t)v;
-    const int top = (int)(__float_as_uint(__uint2float_rz(h)) >> 23) - 127;  // leading bit of h
-    const uint64_t m = (((uint64_t)h << 32) | l) << ((31 - top) & 63);         // leading bit at 63
-    const uint64_t mant = ((m >> 10) + 1) >> 1;  // 53 bits; their leading 1 adds 1 to the exponent field
-    const uint32_t e = (uint32_t)(1022 + (low ? 0 : 32) + top - q);
-    return __hiloint2double((int)((sign | (e << 20)) + hi32(mant)), (int)(uint32_t)mant);
+// (v + rest 2^-32) 2^-q as a double, rounded to nearest (ties up); v in two's
+// complement, |v| < 2^63.  JUMP: the rare leading zero words are skipped in a
+// loop (fewer instructions), else by selections (shorter chain).  (An early
+// return with FP64 instructions would be turned into selections that every call
+// pays for.)
+template <bool JUMP>
+__device__ __forceinline__ double sum_to_double(int64_t v, uint32_t rest, int q) {
+    const uint32_t sign = hi32((uint64_t)v) & 0x80000000u, flip = (uint32_t)((int32_t)sign >> 31);
+    uint32_t c = (rest ^ flip) - flip;  // -(v + rest) = ~v + (1 - rest), or -v
+    const uint64_t m = ((uint64_t)v ^ (((uint64_t)flip << 32) | flip)) + (c == 0 ? flip & 1u : 0u);
+    uint32_t a = hi32(m), b = (uint32_t)m;
+    int e = 1085 - q;
+    if constexpr (JUMP) {
+#pragma unroll 1
+        for (; a == 0 && (b | c) != 0; e -= 32) {
+            a = b;
+            b = c;
+            c = 0;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const bool shift = a == 0;
+            a = shift ? b : a;
+            b = shift ? c : b;
+            c = shift ? 0u : c;
+            e -= shift ? 32 : 0;
+        }
+    }
+    const int up = 31 - leading_bit(a | (a == 0));
+    const uint32_t mh = __funnelshift_l(b, a, up), ml = __funnelshift_l(c, b, up);
+    // 53 bits of the 64 from the leading one on, which adds 1 to the exponent field
+    const uint64_t mant = ((((uint64_t)mh << 32) | ml) >> 11) + ((ml >> 10) & 1u);
+    const uint32_t hi = sign + ((uint32_t)(e - up) << 20) + hi32(mant);
+    return __hiloint2double(a == 0 ? 0 : (int)hi, (int)(uint32_t)mant);
+}
+
+// |v| <= 1, in Q60, rounded down; hi, lo: its words.
+__device__ __forceinline__ uint64_t to_q60(uint32_t hi, uint32_t lo) {
+    const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    return (m << 8) >> min(1023u - ((hi >> 20) & 0x7ffu), 63u);
 }
 
 // Cosine and sine of an angle of a quadrant, with their distance from an axis

@@ -165,3 +165,37 @@ def worst(program):
 @pytest.mark.parametrize("what,bound", [("phases", 2.25), ("radius", 0.5), ("normals", 3.0)])
 def test_errors_relative_to_the_result(worst, what, bound):
     assert worst(what) <= bound
+
+
+SUMS = r"""
+using namespace sdeb;
+// t 2^-60 as a double, rounded to nearest (ties away from 0)
+static double exact(__int128 t) {
+    unsigned __int128 m = t < 0 ? -(unsigned __int128)t : (unsigned __int128)t;
+    int n = 0;
+    while (m >> n >> 53) ++n;
+    if (n) m = (m + ((unsigned __int128)1 << (n - 1))) >> n;
+    return (t < 0 ? -1 : 1) * std::ldexp((double)(uint64_t)m, n - 60);
+}
+int main() {
+    std::mt19937_64 g(5);
+    for (long i = 0; i < 2000000; ++i) {
+        __int128 t = (__int128)(((unsigned __int128)g() << 64) | g()) >> (59 + g() % 69);  // at most 2^68
+        if (i < 200) t = i - 100;
+        const int64_t v = (int64_t)(t >> 6);
+        const uint32_t rest = ((uint32_t)t & 63u) << 26;
+        if (sum_to_double<true>(v, rest, 54) != exact(t) || sum_to_double<false>(v, rest, 54) != exact(t)) return 1;
+    }
+    for (long i = 0; i < 500000; ++i) {
+        double x = std::exp2(-std::uniform_real_distribution<double>(0, 70)(g));
+        const double ends[4] = {0.0, 1.0, 5e-324, 0x1p-60};
+        if (i < 4) x = ends[i];
+        if (to_q60((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x)) != (uint64_t)std::ldexp(x, 60)) return 2;
+    }
+    return 0;
+}
+"""
+
+
+def test_sums_to_double_and_back(program):
+    program(SUMS)()
