@@ -416,10 +416,22 @@ __device__ __forceinline__ void rk4_step(M &model, Real (&x)[M::U][P], Real (&cp
 #pragma unroll
         for (int i = 0; i < P; ++i) acc[c][i] = Real(0);
     model.stage_base(x, cp, base);
-    rk4_stage<M, Real, P>(model, base, base, u0, units, reduce, acc, y, Real(1), Real(0.5));
-    rk4_stage<M, Real, P>(model, y, base, u0, units, reduce, acc, y, Real(2), Real(0.5));
-    rk4_stage<M, Real, P>(model, y, base, u0, units, reduce, acc, y, Real(2), Real(1));
-    rk4_stage<M, Real, P>(model, y, base, u0, units, reduce, acc, y, Real(1), Real(0));
+    if constexpr (M::kFixedSums) {
+        // one stage's code, not four: they would not fit the instruction cache
+#pragma unroll
+        for (int c = 0; c < M::U; ++c)
+#pragma unroll
+            for (int i = 0; i < P; ++i) y[c][i] = base[c][i];
+#pragma unroll 1
+        for (int stage = 0; stage < 4; ++stage)
+            rk4_stage<M, Real, P>(model, y, base, u0, units, reduce, acc, y, stage == 1 || stage == 2 ? Real(2) : Real(1),
+                                  stage < 2 ? Real(0.5) : Real(1));
+    } else {
+        rk4_stage<M, Real, P>(model, base, base, u0, units, reduce, acc, y, Real(1), Real(0.5));
+        rk4_stage<M, Real, P>(model, y, base, u0, units, reduce, acc, y, Real(2), Real(0.5));
+        rk4_stage<M, Real, P>(model, y, base, u0, units, reduce, acc, y, Real(2), Real(1));
+        rk4_stage<M, Real, P>(model, y, base, u0, units, reduce, acc, y, Real(1), Real(0));
+    }
 #pragma unroll
     for (int i = 0; i < P; ++i)
 #pragma unroll
