@@ -273,7 +273,9 @@ SDEB_API sdeb_status sdeb_create_user(const sdeb_problem *pb, const char *source
  * integrate call (sdeb_integrate, sdeb_integrate_range; counted from 0 over
  * the process, sdeb_autotune's trial launches not counted) fail without
  * launching, so the integrate call returns SDEB_ECUDA with the step counter
- * unchanged.  Unset or any other value: no injection. */
+ * unchanged; "trial:<k>" makes the k-th trial of the batch tuner (counted from
+ * 0 over the process) fail, so sdeb_autotune returns SDEB_ECUDA and the batch
+ * keeps its schedule.  Unset or any other value: no injection. */
 
 /* Free the context and its device buffers (synchronises the device first).
  * NULL is accepted. */

@@ -60,8 +60,8 @@ struct sdeb_ctx {
     int *d_head = nullptr;
     int32_t ntasks = 0, team_items = 0;
     int grid = 0;
-    bool grid_tuned = false;              // grid_cap is the tuner's choice
-    int grid_cap = 1;                     // resident blocks of the batch kernel on this device
+    int grid_limit = 1;                   // resident blocks of the batch kernel on this device
+    int grid_choice = 0;                  // those the tuner chose (0: upload_plan's rule)
     cudaStream_t capture_stream = nullptr;
     cudaGraphExec_t graph = nullptr;
     bool batch_done = false;
@@ -106,17 +106,19 @@ struct NvtxRange {
 // buffers in this process (counted from 0) fail as out of memory,
 // "launch:<k>" makes the k-th forward launch of an integrate call
 // (sdeb_integrate, sdeb_integrate_range) fail without launching; the layout
-// tuner's trial launches are not counted.  Read once, at the first
-// allocation or launch; any other value injects nothing.
+// tuner's trial launches are not counted; "trial:<k>" makes the k-th trial of
+// the batch tuner fail.  Read once, at the first allocation or launch; any
+// other value injects nothing.
 struct FaultPlan {
-    long alloc_at = -1, launch_at = -1;
-    std::atomic<long> allocs{0}, launches{0};
+    long alloc_at = -1, launch_at = -1, trial_at = -1;
+    std::atomic<long> allocs{0}, launches{0}, trials{0};
     FaultPlan() {
         const char *v = std::getenv("SDEB_FAULT");
         if (!v) return;
         long k = -1;
         if (std::sscanf(v, "alloc:%ld", &k) == 1 && k >= 0) alloc_at = k;
         else if (std::sscanf(v, "launch:%ld", &k) == 1 && k >= 0) launch_at = k;
+        else if (std::sscanf(v, "trial:%ld", &k) == 1 && k >= 0) trial_at = k;
     }
 };
 
@@ -133,6 +135,11 @@ bool inject_alloc_fault() {
 bool inject_launch_fault() {
     FaultPlan &f = fault_plan();
     return f.launch_at >= 0 && f.launches.fetch_add(1) == f.launch_at;
+}
+
+bool inject_trial_fault() {
+    FaultPlan &f = fault_plan();
+    return f.trial_at >= 0 && f.trials.fetch_add(1) == f.trial_at;
 }
 
 bool model_shape(int32_t model, int32_t n, int32_t &m, int32_t &d, int32_t &units) {
@@ -487,27 +494,34 @@ BatchPlan plan_batch(const std::vector<BatchInstance> &inst, double chain_frac, 
     return plan;
 }
 
-// Upload a plan into the context's tables (sized for the largest plan).
+// Upload a plan into tables of its own; if that fails the context keeps the
+// tables it has.
 sdeb_status upload_plan(sdeb_ctx *c, const BatchPlan &plan) {
-    cudaFree(c->d_items);
-    cudaFree(c->d_tasks);
-    c->d_items = nullptr;
-    c->d_tasks = nullptr;
-    cudaError_t e = cudaMalloc((void **)&c->d_items, sizeof(BatchItem) * std::max<size_t>(1, plan.items.size()));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_tasks, sizeof(BatchTask) * std::max<size_t>(1, plan.tasks.size()));
+    BatchItem *items = nullptr;
+    BatchTask *tasks = nullptr;
+    cudaError_t e = cudaMalloc((void **)&items, sizeof(BatchItem) * std::max<size_t>(1, plan.items.size()));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&tasks, sizeof(BatchTask) * std::max<size_t>(1, plan.tasks.size()));
     if (e == cudaSuccess)
-        e = cudaMemcpy(c->d_items, plan.items.data(), sizeof(BatchItem) * plan.items.size(), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(items, plan.items.data(), sizeof(BatchItem) * plan.items.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = cudaMemcpy(c->d_tasks, plan.tasks.data(), sizeof(BatchTask) * plan.tasks.size(), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(tasks, plan.tasks.data(), sizeof(BatchTask) * plan.tasks.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
+        cudaFree(items);
+        cudaFree(tasks);
         cudaGetLastError();
         return cuda_fail(c, e, "batch plan upload");
     }
+    cudaFree(c->d_items);
+    cudaFree(c->d_tasks);
+    c->d_items = items;
+    c->d_tasks = tasks;
     c->ntasks = (int32_t)plan.tasks.size();
     c->team_items = plan.team_items;
     c->inst_layout = plan.inst_layout;
-    int cap = c->grid_cap;
-    if (c->elem == 4 && !c->grid_tuned) {
+    int cap = c->grid_limit;
+    if (c->grid_choice > 0) {
+        cap = std::min(cap, c->grid_choice);
+    } else if (c->elem == 4) {
         const int sms = std::max(1, c->num_sms);
         cap = std::min(cap, sms * plan_residency(plan, sms, std::max(1, cap / sms)));
     }
@@ -594,18 +608,18 @@ sdeb_status autotune_batch(sdeb_ctx *c, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaMalloc((void **)&tf, (size_t)c->batch_items);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    const int choice_before = c->grid_choice;
     double best_frac = c->batch_chain_frac;
-    int best_grid = c->grid_cap;
+    int best_grid = 0;
     float best_ms = 1e30f;
     bool first = true;
-    const int cap = c->grid_cap;
-    c->grid_tuned = true;
+    const int cap = c->grid_limit;
     for (double frac : {0.125, 0.18, 0.25, 0.35, 0.5, 0.7, 1.0, 2.0})
       for (int per_sm : {1, 2, 3, 4, 5}) {
         if (e != cudaSuccess) break;
         if (per_sm > 1 && per_sm * c->num_sms > cap) break;
-        c->grid_cap = std::min(cap, per_sm * c->num_sms);
-        if (upload_plan(c, plan_batch(c->inst, frac, c->num_sms)) != SDEB_OK) {
+        c->grid_choice = std::min(cap, per_sm * c->num_sms);
+        if (inject_trial_fault() || upload_plan(c, plan_batch(c->inst, frac, c->num_sms)) != SDEB_OK) {
             e = cudaErrorUnknown;
             break;
         }
@@ -624,19 +638,21 @@ sdeb_status autotune_batch(sdeb_ctx *c, cudaStream_t s) {
         if (e == cudaSuccess && ms < best_ms) {
             best_ms = ms;
             best_frac = frac;
-            best_grid = c->grid_cap;
+            best_grid = c->grid_choice;
         }
       }
-    c->grid_cap = best_grid;
     cudaFree(tx);
     cudaFree(tc);
     cudaFree(tf);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    if (e != cudaSuccess) {
+    if (e != cudaSuccess) {  // back to the schedule from before
         cudaGetLastError();
+        c->grid_choice = choice_before;
+        (void)upload_plan(c, plan_batch(c->inst, c->batch_chain_frac, c->num_sms));
         return cuda_fail(c, e, "batch autotune");
     }
+    c->grid_choice = best_grid;
     c->batch_chain_frac = best_frac;
     return upload_plan(c, plan_batch(c->inst, best_frac, c->num_sms));
 }
@@ -1438,7 +1454,7 @@ sdeb_status sdeb_create_batch(const sdeb_problem *pbs, int32_t count, sdeb_ctx *
         return st;
     }
     c->num_sms = sms > 0 ? sms : 1;
-    c->grid_cap = c->num_sms * batch_blocks_per_sm(c->elem == 8);
+    c->grid_limit = c->num_sms * batch_blocks_per_sm(c->elem == 8);
     sdeb_status st = upload_plan(c, plan_batch(c->inst, c->batch_chain_frac, c->num_sms));
     if (st != SDEB_OK) {
         free_buffers(c);
