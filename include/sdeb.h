@@ -391,7 +391,10 @@ SDEB_API sdeb_status sdeb_frames_device_ptr(sdeb_ctx *ctx, void **ptr, size_t *b
  * integration after sdeb_set_params (ESTATE otherwise) and kept for the
  * adjoint.  EINVAL if lanes x units does not cover the orbit's units,
  * EUNSUPPORTED if the model has no kernel for that layout.  sdeb_create
- * picks a default; sdeb_autotune times the candidates. */
+ * picks a default; sdeb_autotune times the candidates.  A context left at its
+ * default runs on the lanes that suit the launch: the Euler-Maruyama kernels
+ * of the phase models take more lanes per orbit in FP64 and for few orbits,
+ * with the default layout's results bit for bit. */
 SDEB_API sdeb_status sdeb_set_layout(sdeb_ctx *ctx, int32_t lanes_per_orbit, int32_t units_per_lane);
 
 /* The checkpoint interval a context keeps (0 without checkpoints, and for a
@@ -411,13 +414,15 @@ SDEB_API sdeb_status sdeb_set_layout(sdeb_ctx *ctx, int32_t lanes_per_orbit, int
  * twice that, with the compensation words).  Gradients do not depend on the
  * interval beyond rounding. */
 SDEB_API sdeb_status sdeb_get_checkpoint_interval(const sdeb_ctx *ctx, int64_t *steps);
+/* The layout asked for by sdeb_set_layout or chosen by sdeb_autotune, else the
+ * default. */
 SDEB_API sdeb_status sdeb_get_layout(const sdeb_ctx *ctx, int32_t *lanes_per_orbit, int32_t *units_per_lane);
 
 /* Layout tuner (motivated by the hand-tuned work-group sizes of the paper's
  * Table 4): times the forward kernel over the first trial_steps steps
  * (<= 0: 64) for every instantiated layout that covers the orbit's units
- * with at most 2x padding, on private copies of the current state, and keeps
- * the fastest.  A context created with ckpt_every > 0 for sdeb_grad is tuned
+ * with at most 2x padding, and for the default left to the launch, on private
+ * copies of the current state, and keeps the fastest.  A context created with ckpt_every > 0 for sdeb_grad is tuned
  * for forward + adjoint instead: both are timed over the first
  * min(ckpt_every, 1024, steps) steps (trial_steps is ignored), the adjoint
  * from checkpoint 0 with a zero dL/dX^K into temporary outputs.  Call after

@@ -757,7 +757,7 @@ cudaError_t dispatch_tuning_layouts(const ForwardArgs &a, Layout l, cudaStream_t
     return dispatch_default_layouts<MF, Real>(a, l, s);
 }
 
-// FP64 phase models: the lanes that a layout's kernel runs on.  The coupling
+// FP64 phase models: the lanes that the default layout runs on.  The coupling
 // sums are exact in fixed point, so a layout's units can go to more lanes
 // with the same results.  4 units per lane instead of 8 or 16 (registers: five
 // resident blocks instead of three), 2 when that leaves less than two warps for
@@ -779,7 +779,7 @@ inline Layout spread_f64(Layout l, int units, int64_t orbits) {
 template <template <typename, int> class MF>
 cudaError_t dispatch_phase_layouts_f64(const ForwardArgs &a, Layout l, cudaStream_t s) {
     using Real = double;
-    l = spread_f64(l, a.units, a.orbits);
+    if (!a.asked) l = spread_f64(l, a.units, a.orbits);
     SDEB_FORWARD_LAYOUT(1, 1)
     SDEB_FORWARD_LAYOUT(1, 2)
     SDEB_FORWARD_LAYOUT(2, 2)
@@ -796,6 +796,20 @@ cudaError_t dispatch_phase_layouts_f64(const ForwardArgs &a, Layout l, cudaStrea
     SDEB_FORWARD_LAYOUT(16, 4)
     SDEB_FORWARD_LAYOUT(32, 4)
     SDEB_FORWARD_LAYOUT(32, 8)
+    return cudaErrorNotSupported;
+}
+
+// The layouts that only run when they are asked for.
+template <template <typename, int> class MF>
+cudaError_t dispatch_asked_layouts_f64(const ForwardArgs &a, Layout l, cudaStream_t s) {
+    using Real = double;
+    SDEB_FORWARD_LAYOUT(1, 8)
+    SDEB_FORWARD_LAYOUT(2, 8)
+    SDEB_FORWARD_LAYOUT(4, 8)
+    SDEB_FORWARD_LAYOUT(8, 8)
+    SDEB_FORWARD_LAYOUT(16, 8)
+    SDEB_FORWARD_LAYOUT(4, 16)
+    SDEB_FORWARD_LAYOUT(8, 16)
     return cudaErrorNotSupported;
 }
 

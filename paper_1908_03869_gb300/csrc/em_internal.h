@@ -60,6 +60,7 @@ struct ForwardArgs {
     int32_t milstein;  // 1: Milstein step (models with multiplicative noise), 0: Euler-Maruyama
     int32_t rk4;       // 1: fourth-order Runge-Kutta on the drift alone (launch_forward_rk4_*)
     int32_t implicit;  // 1: implicit Euler, 2: implicit midpoint on the drift alone (launch_forward_implicit_*)
+    int32_t asked;     // 1: the layout was asked for and runs as it is (else the launch may take other lanes)
     int32_t final_value;  // 1: leave the state's value x - c in x at k_end (no later resume)
     int64_t nckpt;         // checkpoints in ckpt
     unsigned long long *check;  // bounds-check status word (checked build), or null
@@ -90,6 +91,7 @@ cudaError_t launch_state_reset(const void *x, size_t bytes, void *frame0, void *
 // (model, precision, layout) combination has no instantiation.
 cudaError_t launch_forward_kuramoto_f32(const ForwardArgs &a, Layout l, cudaStream_t s);
 cudaError_t launch_forward_kuramoto_f64(const ForwardArgs &a, Layout l, cudaStream_t s);
+cudaError_t launch_forward_kuramoto_f64_asked(const ForwardArgs &a, Layout l, cudaStream_t s);
 cudaError_t launch_forward_other_f32(const ForwardArgs &a, Layout l, cudaStream_t s);
 cudaError_t launch_forward_other_f64(const ForwardArgs &a, Layout l, cudaStream_t s);
 cudaError_t launch_forward_rk4_f32(const ForwardArgs &a, Layout l, cudaStream_t s);
@@ -98,9 +100,9 @@ cudaError_t launch_forward_implicit_f32(const ForwardArgs &a, Layout l, cudaStre
 cudaError_t launch_forward_implicit_f64(const ForwardArgs &a, Layout l, cudaStream_t s);
 // Few orbits of the phase models (Euler-Maruyama): cudaErrorNotSupported, and
 // nothing launched, when the launch is not small enough, keeps checkpoints or
-// has another layout than the default one.
-cudaError_t launch_forward_split_f32(const ForwardArgs &a, Layout l, cudaStream_t s);
-cudaError_t launch_forward_split_f64(const ForwardArgs &a, Layout l, cudaStream_t s);
+// has a layout that was asked for.
+cudaError_t launch_forward_split_f32(const ForwardArgs &a, cudaStream_t s);
+cudaError_t launch_forward_split_f64(const ForwardArgs &a, cudaStream_t s);
 
 // The forward launch of a problem: Runge-Kutta, implicit, phase models or the others.
 inline cudaError_t launch_forward_any(const ForwardArgs &a, Layout l, bool fp64, cudaStream_t s) {
@@ -108,7 +110,7 @@ inline cudaError_t launch_forward_any(const ForwardArgs &a, Layout l, bool fp64,
     if (a.implicit) return fp64 ? launch_forward_implicit_f64(a, l, s) : launch_forward_implicit_f32(a, l, s);
     const bool phase = a.model == kKuramoto || a.model == kKuramotoPaper;
     if (phase) {
-        const cudaError_t e = fp64 ? launch_forward_split_f64(a, l, s) : launch_forward_split_f32(a, l, s);
+        const cudaError_t e = fp64 ? launch_forward_split_f64(a, s) : launch_forward_split_f32(a, s);
         if (e != cudaErrorNotSupported) return e;
     }
     if (phase) return fp64 ? launch_forward_kuramoto_f64(a, l, s) : launch_forward_kuramoto_f32(a, l, s);

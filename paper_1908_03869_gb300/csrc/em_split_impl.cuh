@@ -243,12 +243,9 @@ cudaError_t launch_split(const ForwardArgs &a, cudaStream_t s) {
 // (n = 2 in FP32 crosses between 2^14, 44 / 52, and 2^15, 64 / 52).  So: two
 // warps of consumers for every sub-partition of the GPU in FP64, one in FP32,
 // and in FP32 not past 128 units, where a lane has its eight units in either
-// kernel (n = 256: 99 / 95).  The default layout only: one that was asked for
-// runs as asked.
-inline bool use_split(const ForwardArgs &a, Layout l, bool fp64) {
-    Layout plain{0, 0};
-    if (!default_layout(a.units, plain) || plain.G != l.G || plain.P != l.P) return false;
-    if (a.ckpt != nullptr || a.nckpt > 0 || (!fp64 && a.units > 128)) return false;
+// kernel (n = 256: 99 / 95).  A layout that was asked for runs as asked.
+inline bool use_split(const ForwardArgs &a, bool fp64) {
+    if (a.asked || a.ckpt != nullptr || a.nckpt > 0 || (!fp64 && a.units > 128)) return false;
     int64_t lanes = 1;
     while (lanes < a.units && (fp64 || lanes < 32)) lanes *= 2;
     return a.orbits <= (int64_t)kNumSms * 4 * 32 * (fp64 ? 2 : 1) / lanes;

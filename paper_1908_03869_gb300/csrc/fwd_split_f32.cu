@@ -3,8 +3,8 @@
 
 namespace sdeb {
 
-cudaError_t launch_forward_split_f32(const ForwardArgs &a, Layout l, cudaStream_t s) {
-    if (!use_split(a, l, false)) return cudaErrorNotSupported;
+cudaError_t launch_forward_split_f32(const ForwardArgs &a, cudaStream_t s) {
+    if (!use_split(a, false)) return cudaErrorNotSupported;
     if (a.model == kKuramoto) return launch_split<KuramotoScalarLane, float>(a, s);
     return launch_split<KuramotoPaperLane, float>(a, s);
 }

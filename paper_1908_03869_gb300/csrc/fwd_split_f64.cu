@@ -3,8 +3,8 @@
 
 namespace sdeb {
 
-cudaError_t launch_forward_split_f64(const ForwardArgs &a, Layout l, cudaStream_t s) {
-    if (!use_split(a, l, true)) return cudaErrorNotSupported;
+cudaError_t launch_forward_split_f64(const ForwardArgs &a, cudaStream_t s) {
+    if (!use_split(a, true)) return cudaErrorNotSupported;
     if (a.model == kKuramoto) return launch_split<KuramotoScalarLane, double>(a, s);
     return launch_split<KuramotoPaperLane, double>(a, s);
 }

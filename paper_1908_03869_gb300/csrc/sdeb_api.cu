@@ -28,6 +28,7 @@ struct sdeb_ctx {
     size_t elem = 0;          // 4 or 8
     int device = 0;
     Layout layout{1, 1};
+    bool layout_asked = false;    // by sdeb_set_layout or the tuner; else the default, run on the lanes that suit it
     void *d_params = nullptr;
     size_t params_bytes = 0;
     void *d_x = nullptr;
@@ -1013,6 +1014,7 @@ sdeb_status sdeb_integrate_range(sdeb_ctx *ctx, int64_t k_begin, int64_t k_end, 
     a.milstein = (ctx->pb.flags & SDEB_FLAG_MILSTEIN) ? 1 : 0;
     a.rk4 = (ctx->pb.flags & SDEB_FLAG_RK4) ? 1 : 0;
     a.implicit = implicit_kind(ctx->pb.flags);
+    a.asked = ctx->layout_asked ? 1 : 0;
     cudaError_t e = launch_forward(a, ctx->layout, ctx->pb.precision == SDEB_FP64, as_stream(stream));
     if (e == cudaErrorNotSupported)
         return fail(ctx, SDEB_EUNSUPPORTED, "no kernel for model %d with layout G=%d P=%d", a.model,
@@ -1181,6 +1183,7 @@ sdeb_status sdeb_set_layout(sdeb_ctx *ctx, int32_t lanes_per_orbit, int32_t unit
     if (!layout_instantiated(ctx->pb.model, {G, P}))
         return fail(ctx, SDEB_EUNSUPPORTED, "no kernel for model %d with G=%d P=%d", ctx->pb.model, G, P);
     ctx->layout = {G, P};
+    ctx->layout_asked = true;
     return SDEB_OK;
 }
 
@@ -1207,7 +1210,8 @@ sdeb_status sdeb_autotune(sdeb_ctx *ctx, int64_t trial_steps, void *stream) {
                                                       ctx->ckpt_int);
         adj_steps = std::min<int64_t>(segs * ctx->ckpt_int, ctx->pb.steps);
     }
-    static const Layout kCandidates[] = {{1, 1}, {1, 2}, {1, 4}, {1, 8}, {2, 4}, {2, 8}, {4, 4}, {4, 8}, {4, 16},
+    // {0, 0}: the default layout left to the launch, on the lanes that suit it
+    static const Layout kCandidates[] = {{0, 0}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {2, 4}, {2, 8}, {4, 4}, {4, 8}, {4, 16},
                                          {8, 4}, {8, 8}, {8, 16}, {16, 4}, {16, 8}, {32, 4}, {32, 8}};
     const cudaStream_t s = as_stream(stream);
     const size_t state_bytes = (size_t)ctx->pb.orbits * ctx->pb.n * ctx->elem;
@@ -1224,10 +1228,14 @@ sdeb_status sdeb_autotune(sdeb_ctx *ctx, int64_t trial_steps, void *stream) {
     if (e == cudaSuccess && tune_adjoint) e = cudaMalloc(&t_dp, (size_t)ctx->pb.orbits * ctx->pb.d * ctx->elem);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
-    Layout best = ctx->layout;
+    Layout best = ctx->layout, plain;
+    default_layout(ctx->units, plain);
+    bool best_asked = ctx->layout_asked;
     float best_ms = 1e30f;
-    for (const Layout &l : kCandidates) {
+    for (const Layout &cand : kCandidates) {
         if (e != cudaSuccess) break;
+        const bool asked = cand.G > 0;
+        const Layout l = asked ? cand : plain;
         // lanes x units must cover the orbit and waste at most half of it
         const int64_t cover = (int64_t)l.G * l.P;
         if (cover < ctx->units || (cover > 4 && cover > 2 * (int64_t)ctx->units)) continue;
@@ -1253,6 +1261,7 @@ sdeb_status sdeb_autotune(sdeb_ctx *ctx, int64_t trial_steps, void *stream) {
         a.milstein = (ctx->pb.flags & SDEB_FLAG_MILSTEIN) ? 1 : 0;
         a.rk4 = (ctx->pb.flags & SDEB_FLAG_RK4) ? 1 : 0;
         a.implicit = implicit_kind(ctx->pb.flags);
+        a.asked = asked ? 1 : 0;
         float ms = 0.0f;
         for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {  // the first run warms up
             e = cudaMemcpyAsync(tx, ctx->d_x, state_bytes, cudaMemcpyDeviceToDevice, s);
@@ -1313,6 +1322,7 @@ sdeb_status sdeb_autotune(sdeb_ctx *ctx, int64_t trial_steps, void *stream) {
         if (e == cudaSuccess && ms < best_ms) {
             best_ms = ms;
             best = l;
+            best_asked = asked;
         }
     }
     cudaFree(tx);
@@ -1327,6 +1337,7 @@ sdeb_status sdeb_autotune(sdeb_ctx *ctx, int64_t trial_steps, void *stream) {
         return cuda_fail(ctx, e, "sdeb_autotune");
     }
     ctx->layout = best;
+    ctx->layout_asked = best_asked;
     return SDEB_OK;
 }
 
