@@ -324,16 +324,19 @@ struct FhnLane {
     static constexpr bool kNoise = true;
     static constexpr bool kSplitNoise = false;
     static constexpr bool kDelayedComp = false;
-    // FP32: two units an instruction (pairs of em_device.cuh), with the noise
-    // inside the bracket that dt multiplies:
-    //   dv = dt (v (sigma / sqrt(dt) N - c - v^2 / 3) + v - w + I + c mean)
-    //   dw = eps dt (v + a - b w)
-    // (Milstein: N + sigma sqrt(dt) (N^2 - 1) / 2 for N).  Ten packed operations
-    // a pair of units.  (Polynomials with dt inside every coefficient take
-    // seven, but the coefficients' roundings then add up over the horizon:
-    // 4.7e-8 from the 64-bit result where this form and the scalar one have 3e-8.)
+    // FP32: two units an instruction (pairs of em_device.cuh), the drift and the
+    // noise apart until the last fused multiply-add:
+    //   dv = v (sigma sqrt(dt) N) + dt (v (-c - v^2 / 3) + v - w + I + c mean)
+    //   dw = dt (eps (v + a - b w))
+    // (Milstein: n + n^2 / 2 - sigma^2 dt / 2 for n = sigma sqrt(dt) N).  Twelve
+    // packed operations a pair of units.  Ten do with the noise inside the
+    // bracket that dt multiplies and one constant eps dt; but the bracket then
+    // rounds by the noise over dt (and leaves the range for a small dt), and v
+    // and w run on clocks rounded differently: 2 to 6 % further from the 64-bit
+    // result than the scalar step at dt = 0.01.  (Polynomials with dt inside every
+    // coefficient take seven and are half as far off again.)
     static constexpr bool kPacked = sizeof(Real) == 4 && P > 1;
-    Real kc, kmean, kgsq, kepsdt;
+    Real kgsq;
     Real a, b, eps, I, c, gsq, dt, inv_units;
     Real half_gsq2;  // (sigma sqrt(dt))^2 / 2, the Milstein coefficient
 
@@ -348,13 +351,7 @@ struct FhnLane {
 
     __device__ __forceinline__ void load(const Real *p, int, int units, double dt64, double sqdt64) {
         const Real dt_ = (Real)dt64, sqdt = (Real)sqdt64;
-        if constexpr (kPacked) {
-            const double g = (double)p[5] * sqdt64;
-            kgsq = (Real)(g * (double)bm_amp_unit<float>() / dt64);
-            kc = (Real)(-(double)p[4] - (MIL ? 0.5 * g * g / dt64 : 0.0));
-            kmean = (Real)((double)p[4] / units);
-            kepsdt = (Real)((double)p[2] * dt64);
-        }
+        if constexpr (kPacked) kgsq = (Real)((double)p[5] * sqdt64 * (double)bm_amp_unit<float>());
         a = p[0];
         b = p[1];
         eps = p[2];
@@ -404,20 +401,16 @@ struct FhnLane {
     struct Step2 {
         F2 k0;
     };
-    __device__ __forceinline__ Step2 step2(const Real (&red)[NR]) const { return Step2{dup2(fma_r(kmean, red[0], I))}; }
+    __device__ __forceinline__ Step2 step2(const Real (&red)[NR]) const { return Step2{dup2(fma_r(c, mul_r(red[0], inv_units), I))}; }
     __device__ __forceinline__ F2 noise_scaled2(F2 amp) const { return mul2(dup2(kgsq), amp); }
     __device__ __forceinline__ void incr2(int p, const Step2 &st, const Real (&x)[U][P], F2 amp_scaled, F2 trig,
                                           F2 (&inc)[U]) const {
         const F2 v = pair_of<P>(x[0], p), w = pair_of<P>(x[1], p);
-        F2 m = fma2(dup2(Real(-1.0 / 3.0)), mul2(v, v), dup2(kc));
-        if constexpr (MIL) {
-            const F2 n = mul2(amp_scaled, trig);
-            m = fma2(n, fma2(n, dup2(Real(0.5) * dt), dup2(Real(1))), m);
-        } else {
-            m = fma2(amp_scaled, trig, m);
-        }
-        inc[0] = mul2(dup2(dt), fma2(v, m, add2(sub2(st.k0, w), v)));
-        inc[1] = mul2(dup2(kepsdt), fma2(dup2(-b), w, add2(v, dup2(a))));
+        const F2 m = fma2(dup2(Real(-1.0 / 3.0)), mul2(v, v), dup2(-c));
+        F2 n = mul2(amp_scaled, trig);
+        if constexpr (MIL) n = fma2(n, fma2(n, dup2(Real(0.5)), dup2(Real(1))), dup2(-half_gsq2));
+        inc[0] = fma2(n, v, mul2(dup2(dt), fma2(v, m, add2(sub2(st.k0, w), v))));
+        inc[1] = mul2(dup2(dt), mul2(dup2(eps), fma2(dup2(-b), w, add2(v, dup2(a)))));
     }
 
     __device__ __forceinline__ void drift_incr(int i, const Real (&x)[U][P], const Real (&red)[NR],
