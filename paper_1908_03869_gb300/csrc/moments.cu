@@ -59,28 +59,38 @@ __device__ __forceinline__ Acc acc_from_shifted(double cnt, double K, double s1,
     return a;
 }
 
-// s + c += a exactly but for the rounding of c: s takes the rounded sum, c
-// its error (D. E. Knuth's two-sum).
-__device__ __forceinline__ void two_sum_add(float &s, float &c, float a) {
+// s += a, and the error of that sum exactly (D. E. Knuth's two-sum).
+__device__ __forceinline__ float two_sum_add(float &s, float a) {
     const float t = __fadd_rn(s, a);
     const float z = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(a, z)));
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(a, z));
     s = t;
+    return e;
 }
 
-// Elements whose shifted sums are carried as FP32 pairs before they go to the
-// FP64 accumulators.
+// A sum of FP32 terms as three FP32 numbers: the value, the errors of its sums
+// and the errors of theirs.
+struct TripleSum {
+    float a = 0.0f, b = 0.0f, c = 0.0f;
+    __device__ __forceinline__ void add(float x) { add_low(two_sum_add(a, x)); }
+    __device__ __forceinline__ void add_low(float x) { c = __fadd_rn(c, two_sum_add(b, x)); }  // of 2^-24 of the terms' size
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
+// Elements whose shifted sums are carried in FP32 before they go to the FP64
+// accumulators.
 constexpr int kMomGroup = 16;
 
 // s1 += sum (x - K), s2 += sum (x - K)^2 over the elements x[0], x[step], ...
 // (count of them) of one thread.  An SM takes 128 FP32 operations a clock and
-// 1.68 FP64 ones, so FP32 elements are summed as FP32 pairs, kMomGroup at a
-// time: x - K is split exactly into dh + dl, dh^2 into a product and its
-// error, the running sums into a value and the sum of its errors.  A group's
-// sums are off by some 2^-47 of the group; over a chunk's groups these errors
-// average out below those of adding its elements one by one in FP64 (each up
-// to 2^-53 of the whole sum).  25 FP32 operations and half an FP64 one an
-// element instead of 5 FP64 ones.  Elements so far from K (2^60), or all so
+// 1.68 FP64 ones, so FP32 elements are summed as FP32 triples, kMomGroup at a
+// time: x - K is split exactly into dh + dl, and (dh + dl)^2 into terms that
+// drop less than 2^-70 of it.  A group's sums are off by some 2^-66, so the
+// FP64 sums round once a group instead of once an element: at or below the error of
+// adding the elements one by one in FP64.  (With FP32 pairs, 25 operations an
+// element instead of 62, a group is off by 2^-47, and the variance of 64 or
+// 300 orbits was 4 to 20 times further off than with FP64 sums.)  Half an FP64
+// operation an element instead of 5.  Elements so far from K (2^60), or all so
 // near it (2^-40), that a product or its error leaves the FP32 range, and
 // non-finite ones, are taken again in FP64.
 __device__ __forceinline__ void shifted_sums_f64(const float *x, int64_t step, int count, double K, double &s1,
@@ -102,22 +112,25 @@ __device__ __forceinline__ void shifted_sums(const float *x, int64_t step, int c
         float v[kMomGroup];
 #pragma unroll
         for (int i = 0; i < kMomGroup; ++i) v[i] = i0 + i < count ? x[(i0 + i) * step] : Kf;  // past the end: d = 0
-        float a = 0.0f, ac = 0.0f, q = 0.0f, qc = 0.0f;
+        TripleSum sum, sq;
 #pragma unroll
         for (int i = 0; i < kMomGroup; ++i) {
             const float dh = __fsub_rn(v[i], Kf);
             const float z = __fsub_rn(dh, v[i]);
             const float dl = __fsub_rn(__fsub_rn(v[i], __fsub_rn(dh, z)), __fadd_rn(Kf, z));
             far = fmaxf(far, fabsf(dh));
-            const float p = __fmul_rn(dh, dh);
-            const float e = __fmaf_rn(__fadd_rn(dh, dh), dl, __fmaf_rn(dh, dh, -p));
-            two_sum_add(a, ac, dh);
-            ac = __fadd_rn(ac, dl);
-            two_sum_add(q, qc, p);
-            qc = __fadd_rn(qc, e);
+            sum.add(dh);
+            sum.add_low(dl);
+            // (dh + dl)^2 = p + e + c1 + c2: dh^2 and its error, 2 dh dl and its error with dl^2
+            const float p = __fmul_rn(dh, dh), h2 = __fadd_rn(dh, dh);
+            const float c1 = __fmul_rn(h2, dl);
+            sq.add(p);
+            sq.add_low(__fmaf_rn(dh, dh, -p));
+            sq.add_low(c1);
+            sq.c = __fadd_rn(sq.c, __fmaf_rn(dl, dl, __fmaf_rn(h2, dl, -c1)));
         }
-        s1 += (double)a + (double)ac;
-        s2 += (double)q + (double)qc;
+        s1 += sum.value();
+        s2 += sq.value();
     }
     const bool in_range = far == 0.0f || (far >= 0x1p-40f && far <= 0x1p60f);
     if (!in_range || !isfinite(s1) || !isfinite(s2)) shifted_sums_f64(x, step, count, K, s1, s2);
