@@ -66,12 +66,12 @@ FALLBACK_SM_MHZ = 2070.0
 # whitespace left out); a counter is reported only while the fingerprint
 # matches (null once the kernel's code has changed).
 FORWARD_SOURCES = ["em_forward_impl.cuh", "em_device.cuh", "em_models.cuh", "fwd_kuramoto_f32.cu",
-                   "fwd_kuramoto_f64.cu", "em_internal.h"]
+                   "fwd_kuramoto_f64.cu", "em_internal.h", "fixed_math.cuh"]
 NCU_COUNTERS = {
     # DRAM bytes (read + write) of one full-size forward launch of the n = 32 problem
-    "forward_n32_dram_bytes": {"sha": "b58b7a844f81edb6", "value": 3.488e9},
+    "forward_n32_dram_bytes": {"sha": "372b8f248929a0ba", "value": 3.487e9},
     # FP64-pipe thread-instructions per oscillator-step of the FP64 forward kernel
-    "fp64_pipe_inst_per_osc_step": {"sha": "b58b7a844f81edb6", "value": 65.63},
+    "fp64_pipe_inst_per_osc_step": {"sha": "372b8f248929a0ba", "value": 4.57},
 }
 
 

@@ -352,7 +352,7 @@ __device__ __forceinline__ void run_team(const BatchArgs &a, int32_t item, Real 
 // FP32: registers for four resident blocks per SM, no spills (the planner
 // picks one to four; five, on 96 registers with spilled words, were slower on
 // every batch measured: 48 instances x 512 orbits to 1e4 steps 19.3 ms at
-// five, 18.5 at four).  FP64 keeps five (96 per thread, a few spilled words).
+// five, 18.5 at four).  FP64 keeps five (96 per thread, some 86 spilled words).
 template <typename Real>
 __global__ void __launch_bounds__(kBatchBlock, sizeof(Real) == 4 ? 4 : 5) em_batch_kernel(const BatchArgs a) {
     __shared__ int s_task;

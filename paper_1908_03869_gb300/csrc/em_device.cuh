@@ -102,8 +102,9 @@ inline PhiloxKeys philox_key_schedule(uint64_t seed) {
 // (fma.rn.f32x2 and its kin), each half rounded as the scalar instruction
 // rounds it.  Measured: of use where an FP32 kernel is bound by issue slots
 // (the FitzHugh-Nagumo step); the phase kernels, held by the special-function
-// and integer-multiply pipes at the same time, ran from 4 % faster (n = 8) to
-// 5 % slower (n = 128) with it, and stay scalar.
+// and integer-multiply pipes at the same time, ran 3 % faster (n = 8), 3 %
+// slower (n = 32) and 7 % slower (n = 128) with it (5 % with a scalar
+// Box-Muller), and stay scalar.
 // ---------------------------------------------------------------------------
 
 struct F2 {

@@ -759,14 +759,15 @@ cudaError_t dispatch_tuning_layouts(const ForwardArgs &a, Layout l, cudaStream_t
 
 // FP64 phase models: the lanes that the default layout runs on.  The coupling
 // sums are exact in fixed point, so a layout's units can go to more lanes
-// with the same results.  4 units per lane instead of 8 or 16 (registers: five
+// with the same results.  4 units per lane instead of 8 (registers: five
 // resident blocks instead of three), 2 when that leaves less than two warps for
 // every SM sub-partition, on teams of two or four warps past 64 units.
-// Measured, with the fixed-point sums in both: n = 32, 65536 orbits x 200
-// steps 5.95 ms at 4 units (7.8 at 8 with FP64 sums; the FP64, integer
-// multiply and ALU pipes are then 64 to 75 % busy each); n = 100, 64 orbits x
-// 1000 steps 1.43 ms on teams of two warps (5.5 at 8 units, 16 lanes); n = 4,
-// 1024 orbits x 1000 steps 1.29 ms at 2 units (2.5 at 4).
+// Measured, ms, against the layouts as asked for: n = 32, 65536 orbits x 200
+// steps 6.43 at 4 units, 8.64 at 8 (ALU, integer-multiply and FP64 pipes 63,
+// 67 and 48 % busy at 4); 1000 steps of n = 100, 600 orbits 1.95 on teams of two
+// warps, 2.68 at 4 units, 5.96 at 8; of n = 200, 600 orbits 3.30 on teams of four,
+// 5.88 at 8; of n = 8, 10000 orbits 2.42 at 2 units, 3.25 at 4, 5.91 at 8; of
+// n = 4, 20000 orbits 2.43 at 2 units, 3.26 at 4.
 inline Layout spread_f64(Layout l, int units, int64_t orbits) {
     while (l.P > 4 && l.G < 32) l = {l.G * 2, l.P / 2};
     if (l.P >= 4 && units > 2 && orbits * l.G < (int64_t)kNumSms * 4 * 2 * 32) {

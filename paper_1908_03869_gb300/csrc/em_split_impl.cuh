@@ -10,9 +10,10 @@
 // block barrier per kSplitSteps steps hands the halves over.  The results are
 // the bits of the other kernels: FP64 sums are exact, FP32 ones are added in
 // the default layout's order.
-// Measured (before: the whole step on every lane): 1024 orbits of n = 4, FP64,
-// 1000 steps 1.30 -> 0.57 ms a pass; 64 orbits of n = 100, FP64, 1000 steps
-// with moments 1.43 -> 0.90 ms; 256 orbits of n = 8, FP32, 200 steps 82 -> 55 us.
+// Measured, whole passes (before: the whole step on every lane): 1024 orbits of
+// n = 4, FP64, 1000 steps 1.30 -> 0.65 ms; 64 orbits of n = 100, FP64, 1000 steps
+// with moments 1.43 -> 0.97 ms; 256 orbits of n = 8, FP32, 200 steps 77 -> 55 us
+// (45 to 47 with the start state set by one kernel).
 #pragma once
 
 #include "em_forward_impl.cuh"
@@ -237,9 +238,12 @@ cudaError_t launch_split(const ForwardArgs &a, cudaStream_t s) {
 }
 
 // Where the line lies, measured for n = 2 to 256 and 2^8 to 2^17 units in all,
-// 300 steps, this kernel against the others (n = 8; us):
-//   FP64   2^13 units 177 / 388, 2^15 312 / 392, 2^16 502 / 500, 2^17 928 / 814
-//   FP32   2^13 units  48 /  89, 2^14  56 /  89, 2^15  74 /  89, 2^16 122 /  89
+// 300 steps, this kernel against the others (us):
+//   FP64, n = 8   4864 units 202 / 446, 9728 202 / 446, 19456 235 / 443, 38912
+//                 (the line) 381 / 446; n = 2, 64, 256 there 313 / 431, 365 / 459,
+//                 435 / 492; past it, before its sums kept small phases' bits,
+//                 2^16 502 / 500, 2^17 928 / 814
+//   FP32, n = 8   2^13 units  48 /  89, 2^14  56 /  89, 2^15  74 /  89, 2^16 122 /  89
 // (n = 2 in FP32 crosses between 2^14, 44 / 52, and 2^15, 64 / 52).  So: two
 // warps of consumers for every sub-partition of the GPU in FP64, one in FP32,
 // and in FP32 not past 128 units, where a lane has its eight units in either

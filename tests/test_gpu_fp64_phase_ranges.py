@@ -3,7 +3,7 @@ rest next to 0, phases wound past 2^21) are not much slower than those inside.
 65536 orbits of n = 8, 100 steps: Euler-Maruyama 0.93 ms inside, 1.45 at rest,
 1.54 past 2^21; Runge-Kutta 0.81, 1.68 and 1.75 (with CUDA's sincos for every
 phase: 7.5 and 3.46).  The bound leaves a factor of 1.4 over the largest of
-these ratios for a shared machine."""
+these ratios for noise."""
 import pytest
 import torch
 
